@@ -594,7 +594,7 @@ int schedule_many(fb_fft_plan_s* p, TwiddleBuilder& twb)
         if (L <= FB_FFT_MAX_SMEM_LEN && !via_fourstep) {
             PassPlan q;
             int rc = make_line_pass(q, twb, L, 1, (long long)idx.size(), 1, L, 0, 1, L, 0, false, false, false,
-                                    p->odd_first, p->max_lines);
+                                    p->odd_first, p->max_lines, false, true);
             if (rc != FB_FFT_OK) return rc;
             q.off_in_idx = q.off_out_idx = push_offsets(0, idx.size());
             if (!pow2) q.async_ok = false;  // the generic kernel copies offset-table tiles itself
@@ -623,7 +623,8 @@ int schedule_many(fb_fft_plan_s* p, TwiddleBuilder& twb)
             const long long nb = std::min(chunk, cnt - b0);
             const long long at = push_offsets((size_t)b0, (size_t)nb);
             PassPlan a, r;
-            rc = make_line_pass(a, twb, N1, nb, N2, N2, 1, L, N2, 1, L, true, true, true, p->odd_first, p->max_lines);
+            rc = make_line_pass(a, twb, N1, nb, N2, N2, 1, L, N2, 1, L, true, true, true, p->odd_first, p->max_lines,
+                                false, true);
             if (rc != FB_FFT_OK) return rc;
             a.d.ptw_log = plog;
             a.d.ptw_lo = reinterpret_cast<const float2*>(lo_off);
@@ -635,7 +636,7 @@ int schedule_many(fb_fft_plan_s* p, TwiddleBuilder& twb)
             a.group = 1;
             a.slot = slot;
             rc = make_line_pass(r, twb, N2, nb, N1, 1, N2, L, N1, 1, L, false, true, false, p->odd_first,
-                                p->max_lines);
+                                p->max_lines, false, true);
             if (rc != FB_FFT_OK) return rc;
             r.off_out_idx = at;
             if ((N2 & (N2 - 1)) != 0) r.async_ok = false;
@@ -928,6 +929,15 @@ int build_plan(fb_fft_plan_s* p)
             q.grid = std::min(q.grid, (long long)ncl * k.cluster);
             q.d.err = p->err;
             q.d.tw = p->tw;
+            continue;
+        }
+        if (q.kind == 5) {  // one tile per CTA: no cap
+            q.d.err = p->err;
+            q.d.tw = p->tw;
+            if (q.d.ptw) {
+                q.d.ptw_lo = p->tw + reinterpret_cast<long long>(q.d.ptw_lo);
+                q.d.ptw_hi = p->tw + reinterpret_cast<long long>(q.d.ptw_hi);
+            }
             continue;
         }
         FB_CK(line_occupancy(k, q.smem, &occ));

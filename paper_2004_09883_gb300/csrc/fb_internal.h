@@ -87,6 +87,11 @@ struct PassDesc {
     int dep_post;
     int dep;
     int dep_need;
+    // Composite-radix kernels (fft_mr.cuh): lines per tile, and
+    // ceil(2^32 / tiles_per_o) where that divides a tile number below 2^32
+    // (0: one outer index, or 64-bit numbers).
+    int T;
+    unsigned tpo_mag;
 };
 
 // Fill ns[] (product of the earlier radices) and its multiply-high
@@ -142,7 +147,8 @@ inline size_t line_smem_bytes(long long land_elems, int L, int T, int nst, bool 
 
 // One compiled line-pass kernel.  kind 0: compile-time power-of-two kernel
 // (lg = log2 L, io = its IoMode); 1: generic kernel; 2: mixed kernel
-// (lg = log2 of L's power-of-two factor); 3: plane pass (lg1 = log2 rows,
+// (lg = log2 of L's power-of-two factor); 5: composite-radix kernel (lg = L,
+// io = its IoMode); 3: plane pass (lg1 = log2 rows,
 // lg = log2 row length, launched in clusters of `cluster` CTAs).
 struct LineKernel {
     void (*fn)(LineArgs);
@@ -174,6 +180,8 @@ long long plane_smem_bytes(int lg1, int lg2, int threads);
 // Clusters of a cluster kernel that fit the GPU at once.
 cudaError_t line_cluster_occupancy(const LineKernel& k, size_t smem, int* clusters);
 LineKernel line_kernel_mixed(bool forward, int lg2);
+// Composite-radix pass (fft_mr.cuh) of L points, io = its IoMode.
+LineKernel line_kernel_mr(bool forward, int L, int io);
 // Raise a kernel's dynamic shared-memory limit to the device's opt-in maximum,
 // once per (kernel, device); split_regs > 0 also checks the kernel's register
 // count (see LineKernel::split_regs).

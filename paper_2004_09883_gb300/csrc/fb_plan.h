@@ -18,6 +18,7 @@
 #include "fb_fft.h"
 #include "fb_internal.h"
 #include "fft_p2.cuh"
+#include "mr_config.h"
 
 namespace fbfft {
 namespace plan {
@@ -37,6 +38,10 @@ inline int nn_small_threads(long long L)
     return v ? v : (L <= 128 ? 64 : 128);
 }
 
+// Contiguous composite-radix tiles hold fewer lines where a pass would
+// otherwise have fewer tiles than this many per SM of a GB300.
+constexpr int kMrMinTilesPerSm = 2, kMrSms = 152;
+
 enum BufKind { kBufIn = 0, kBufOut = 1, kBufScratch = 2 };
 constexpr size_t kMaxSmemBytes = 227 * 1024;
 
@@ -47,7 +52,7 @@ struct PassPlan {
     int io;       // IoMode of the power-of-two kernel
     int kind;     // 0 power-of-two kernel, 1 generic kernel, 2 mixed kernel (lg = log2 of the 2-factor),
                   // 3 plane pass (two trailing axes, lg1 = log2 rows, lg = log2 row length),
-                  // 4 job of the batched-uneven kernel
+                  // 4 job of the batched-uneven kernel, 5 composite-radix kernel
     int lg1 = 0;
     long long grid;
     size_t smem;
@@ -146,7 +151,7 @@ inline int split_fourstep(long long n, long long* n1, long long* n2)
     return FB_FFT_OK;
 }
 
-// Twiddle tables one line length reads: a table per stage s with Ns > 1
+// Twiddle tables one line length reads: a table per stage s > 0
 // (entries w_{Ns R}^{r k} at [(r-1) Ns + k]) and, for a power-of-two length
 // whose last stage is split (p2_tw_split), the 16 x 15 factor table w_L^{r k},
 // k < 16.  Lays them out from element `base` (each table 16-byte aligned),
@@ -161,7 +166,7 @@ inline long long stage_tables(long long L, const int* radix, int nst, long long 
     for (int s = 0; s <= nst; ++s) off[s] = 0;
     for (int s = 0; s < nst; ++s) {
         const long long cnt = Ns * (radix[s] - 1);
-        if (Ns > 1 && cnt > 0) {
+        if (s > 0 && cnt > 0) {  // (ones where a radix-1 stage came before)
             jobs[(*njobs)++] = TwiddleJob{total, cnt, 0, 0, 1, radix[s], (int)Ns};
             off[s] = (int)total;
             total += (cnt + 1) & ~1LL;
@@ -186,6 +191,7 @@ inline LineKernel pass_kernel(const PassPlan& q, bool fwd)
     }
     if (q.tc) return line_kernel_p2tc(q.threads, fwd, q.lg, q.io);
     if (q.kind == 3) return line_kernel_plane(fwd, q.lg1, q.lg, q.threads);
+    if (q.kind == 5) return line_kernel_mr(fwd, q.d.L, q.io);
     if (q.kind == 2) return line_kernel_mixed(fwd, q.lg);
     if (q.kind == 1) return line_kernel_generic(fwd);
     return line_kernel_p2(q.threads, fwd, q.lg, q.io);
@@ -198,7 +204,7 @@ inline size_t pass_smem(const PassPlan& q, bool async)
     const size_t ptw = q.d.ptw_smem ? (size_t)(ptw_pad((int)((1LL << q.d.ptw_log) + q.d.ptw_hi_cnt - 1)) + 1) * sizeof(float2) : 0;
     if (q.kind == 0) return (size_t)p2_smem_bytes(q.threads, q.lg, q.io, async, q.tc) + ptw;
     if (q.kind == 3) return (size_t)plane_smem_bytes(q.lg1, q.lg, q.threads);
-    if (q.kind == 4) return q.smem;
+    if (q.kind == 4 || q.kind == 5) return q.smem;
     return line_smem_bytes(q.d.land_stride, q.d.L, 1 << q.d.logT, q.d.nst, async, q.d.tws);
 }
 
@@ -228,20 +234,74 @@ inline void ptw_to_smem(PassPlan& a, long long hi_cnt)
     a.smem = smem;
 }
 
+// A line pass of a length with a factor 3 or 5 on the composite-radix kernel
+// (arguments as make_line_pass).
+template <class Twiddles>
+int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long C, long long in_sn, long long in_sc,
+                 long long in_so, long long out_sk, long long out_sc, long long out_so, bool in_tfast, bool out_tfast,
+                 bool ptw)
+{
+    p = PassPlan{};
+    PassDesc& d = p.d;
+    if (in_tfast && !out_tfast) return FB_FFT_ERR_UNSUPPORTED_SIZE;  // never planned
+    p.kind = 5;
+    p.io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
+    if (L < 2 || L > FB_FFT_MAX_SMEM_LEN) return FB_FFT_ERR_UNSUPPORTED_SIZE;
+    const MrConfig c = mr_config((int)L, p.io);
+    if (c.n < 2 || !line_kernel_mr(true, (int)L, p.io).fn) return FB_FFT_ERR_UNSUPPORTED_SIZE;
+    d.L = (int)L;
+    d.nst = c.n;
+    for (int s = 0; s < c.n; ++s) d.radix[s] = c.radix[s];
+    set_stage_products(d);
+    int off[kMaxStages + 1] = {};
+    if (!twb.stages(L, d.radix, d.nst, off)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
+    for (int s = 0; s < d.nst; ++s) d.twoff[s] = off[s];
+    // fewer lines per tile than the kernel's most when that leaves SMs idle
+    // (contiguous lines: the kernel takes any number up to c.T)
+    const long long T =
+        p.io != kIoNN ? c.T : std::max(1LL, std::min<long long>(c.T, C / (kMrMinTilesPerSm * kMrSms)));
+    p.threads = c.threads;
+    d.T = (int)T;
+    d.logT = ilog2ll(T);
+    d.in_sn = in_sn, d.in_sc = in_sc, d.in_so = in_so;
+    d.out_sk = out_sk, d.out_sc = out_sc, d.out_so = out_so;
+    d.C = C;
+    d.tiles_per_o = (C + T - 1) / T;
+    d.ntiles = O * d.tiles_per_o;
+    d.in_tfast = in_tfast ? 1 : 0;
+    d.out_tfast = out_tfast ? 1 : 0;
+    d.ptw = ptw ? 1 : 0;
+    d.scale = 1.0f;
+    d.box_rows = 1;
+    d.tpo_mag = (d.tiles_per_o > 1 && d.ntiles < (1LL << 32))
+                    ? (unsigned)(((1ULL << 32) + d.tiles_per_o - 1) / d.tiles_per_o) : 0u;
+    p.smem = (size_t)(c.buf[0] + c.buf[1] + c.ptw) * sizeof(float2);
+    if (p.smem > kMaxSmemBytes) return FB_FFT_ERR_UNSUPPORTED_SIZE;
+    p.async_ok = false;
+    p.grid = std::min(d.ntiles, 0x7fffffffLL);  // one tile per CTA
+    return FB_FFT_OK;
+}
+
 // Fill a line pass: L-point DFTs over lines (o, c); strides in elements.
 // `twb` receives the stage twiddle tables the pass reads: it provides
 // bool stages(L, radix, nst, off) writing the table offsets of the nst
 // stages, then (off[nst]) that of a split last stage's factor table, and
-// returns false when it has no room for them.
+// returns false when it has no room for them.  per_kernel: the passes of the
+// batched-uneven engine 1, whose tiles go through offset tables.
 template <class Twiddles>
 int make_line_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long C,
                    long long in_sn, long long in_sc, long long in_so, long long out_sk, long long out_sc,
-                   long long out_so, bool in_tfast, bool out_tfast, bool ptw, bool odd_first = false,
-                   int max_lines = 0, bool tc = false)
+                    long long out_so, bool in_tfast, bool out_tfast, bool ptw, bool odd_first = false,
+                   int max_lines = 0, bool tc = false, bool per_kernel = false)
 {
+    const bool pow2_len = (L & (L - 1)) == 0;
+    // lengths with a factor 3 or 5: the composite-radix kernel (66.6 against
+    // 148.4 us on 1000-point lines x 20001, 161 against 694 us on a 120 x 150 x
+    // 144 x 4 volume forward and back); per_kernel keeps the offset-table kernels
+    if (!pow2_len && !per_kernel)
+        return make_mr_pass(p, twb, L, O, C, in_sn, in_sc, in_so, out_sk, out_sc, out_so, in_tfast, out_tfast, ptw);
     p = PassPlan{};  // zero descriptor, default member values (no offset tables)
     PassDesc& d = p.d;
-    const bool pow2_len = (L & (L - 1)) == 0;
     const bool mixed_len = !pow2_len && L <= kMixedMaxLen;  // mixed kernels fix the radix order
     int nst = factorize(L, d.radix, kMaxStages, odd_first && !pow2_len && !mixed_len);
     if (nst < 0) return nst;

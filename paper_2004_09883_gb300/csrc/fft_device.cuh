@@ -27,9 +27,17 @@ namespace fbfft {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
 __device__ __forceinline__ float2 operator+(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 operator-(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+// s * a + b and s * a, s real: one paired instruction each.
+__device__ __forceinline__ float2 fma_real(float s, float2 a, float2 b) { return __ffma2_rn(make_float2(s, s), a, b); }
+__device__ __forceinline__ float2 mul_real(float s, float2 a) { return __fmul2_rn(make_float2(s, s), a); }
 #else
 __host__ __device__ __forceinline__ float2 operator+(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ float2 operator-(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__host__ __device__ __forceinline__ float2 fma_real(float s, float2 a, float2 b)
+{
+    return make_float2(fmaf(s, a.x, b.x), fmaf(s, a.y, b.y));
+}
+__host__ __device__ __forceinline__ float2 mul_real(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
 #endif
 __host__ __device__ __forceinline__ float2 operator*(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
 
@@ -114,26 +122,23 @@ template <bool FWD>
 __host__ __device__ __forceinline__ void dft3(float2& a, float2& b, float2& c)
 {
     const float2 t = b + c;
-    const float2 m = a - 0.5f * t;
-    const float2 d = FB_S3 * mul_si<FWD>(b - c);
+    const float2 m = fma_real(-0.5f, t, a);
+    const float2 d = mul_real(FB_S3, b - c);
     a = a + t;
-    b = m + d;
-    c = m - d;
+    add_sub_si<FWD>(m, d, b, c);  // m +- (s i) d
 }
 
 template <bool FWD>
 __host__ __device__ __forceinline__ void dft5(float2* v)
 {
     const float2 t1 = v[1] + v[4], t2 = v[2] + v[3], t3 = v[1] - v[4], t4 = v[2] - v[3];
-    const float2 a1 = make_float2(v[0].x + FB_C5_1 * t1.x + FB_C5_2 * t2.x, v[0].y + FB_C5_1 * t1.y + FB_C5_2 * t2.y);
-    const float2 a2 = make_float2(v[0].x + FB_C5_2 * t1.x + FB_C5_1 * t2.x, v[0].y + FB_C5_2 * t1.y + FB_C5_1 * t2.y);
-    const float2 b1 = mul_si<FWD>(make_float2(FB_S5_1 * t3.x + FB_S5_2 * t4.x, FB_S5_1 * t3.y + FB_S5_2 * t4.y));
-    const float2 b2 = mul_si<FWD>(make_float2(FB_S5_2 * t3.x - FB_S5_1 * t4.x, FB_S5_2 * t3.y - FB_S5_1 * t4.y));
+    const float2 a1 = fma_real(FB_C5_2, t2, fma_real(FB_C5_1, t1, v[0]));
+    const float2 a2 = fma_real(FB_C5_1, t2, fma_real(FB_C5_2, t1, v[0]));
+    const float2 b1 = fma_real(FB_S5_2, t4, mul_real(FB_S5_1, t3));
+    const float2 b2 = fma_real(-FB_S5_1, t4, mul_real(FB_S5_2, t3));
     v[0] = v[0] + t1 + t2;
-    v[1] = a1 + b1;
-    v[4] = a1 - b1;
-    v[2] = a2 + b2;
-    v[3] = a2 - b2;
+    add_sub_si<FWD>(a1, b1, v[1], v[4]);
+    add_sub_si<FWD>(a2, b2, v[2], v[3]);
 }
 
 // 8 = 2 x 4: even/odd 4-point DFTs, then Y[k] = E[k] +- w8^k O[k].

@@ -44,6 +44,29 @@ LineKernel line_kernel_p2(int threads, bool forward, int lg, int io)
     return none;
 }
 
+#define FB_MR_DECL(IO)                          \
+    LineKernel line_kernel_mr_fwd_##IO##_a(int L); \
+    LineKernel line_kernel_mr_fwd_##IO##_b(int L); \
+    LineKernel line_kernel_mr_inv_##IO##_a(int L); \
+    LineKernel line_kernel_mr_inv_##IO##_b(int L);
+FB_MR_DECL(nn)
+FB_MR_DECL(cc)
+FB_MR_DECL(nc)
+FB_MR_DECL(ccp)
+#undef FB_MR_DECL
+LineKernel line_kernel_mr(bool forward, int L, int io)
+{
+    using Table = LineKernel (*)(int);
+#define FB_MR_TABLES(IO) \
+    {line_kernel_mr_fwd_##IO##_a, line_kernel_mr_fwd_##IO##_b, line_kernel_mr_inv_##IO##_a, line_kernel_mr_inv_##IO##_b}
+    static const Table tables[4][4] = {FB_MR_TABLES(nn), FB_MR_TABLES(cc), FB_MR_TABLES(nc), FB_MR_TABLES(ccp)};
+#undef FB_MR_TABLES
+    LineKernel k{nullptr, 0, false, 0, 0};
+    if (io < 0 || io > 3) return k;
+    for (int half = 0; half < 2 && !k.fn; ++half) k = tables[io][(forward ? 0 : 2) + half](L);
+    return k;
+}
+
 LineKernel line_kernel_p2tc(int threads, bool forward, int lg, int io)
 {
     const LineKernel none{nullptr, 0, false, 0, 0};
@@ -168,6 +191,9 @@ void line_kernel_name(const LineKernel& k, char* buf, size_t n)
     static const char* io_names[4] = {"NN", "CC", "NC", "CCP"};
     if (k.kind == 3)
         snprintf(buf, n, "k_fft_plane<%dx%d,%s>", 1 << k.lg1, 1 << k.lg, k.fwd ? "fwd" : "inv");
+    else if (k.kind == 5)
+        snprintf(buf, n, "k_fft_mr<%d,%s,L=%d,%s>", k.threads, k.fwd ? "fwd" : "inv", k.lg,
+                 (k.io >= 0 && k.io < 4) ? io_names[k.io] : "?");
     else if (k.kind == 2)
         snprintf(buf, n, "k_fft_mixed<%d,%s,2^%d>", k.threads, k.fwd ? "fwd" : "inv", k.lg);
     else if (k.kind == 0)

@@ -1,0 +1,19 @@
+// fft_kernels_mr_fwd_cc_a.cu -- composite-radix line passes, forward:
+// strided lines.
+#include "fft_p2.cuh"
+#include "fft_mr.cuh"
+#include "mr_lengths.h"
+
+namespace fbfft {
+
+LineKernel line_kernel_mr_fwd_cc_a(int L)
+{
+    switch (L) {
+#define FB_MR_CASE(N) \
+    case N: return mr_entry<true, N, kIoCC>();
+        FB_MR_LENGTHS_A(FB_MR_CASE)
+    default: return LineKernel{nullptr, 0, false, 0, 0};
+    }
+}
+
+}  // namespace fbfft
