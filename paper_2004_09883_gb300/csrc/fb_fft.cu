@@ -778,6 +778,20 @@ bool use_plane_pass(const fb_fft_plan_s* p)
     return s && s[0] == '1';
 }
 
+// Four-step pairs of composite-radix passes: columns per tile when the
+// columns may leave the intermediate in their own tiles (each one contiguous
+// block; the rows then read runs of the two tiles' widths multiplied) instead
+// of in rows, of which a column tile would write 32-byte pieces.  0: rows.  Whole
+// tiles only, and the rows' first stage needs its butterflies' inputs a whole
+// number of blocks apart.
+long long fourstep_blocks(long long N1, long long N2)
+{
+    const MrConfig* a = line_kernel_mr(true, (int)N1, kIoCCP).mr;
+    const MrConfig* r = line_kernel_mr(true, (int)N2, kIoNC).mr;
+    if (!a || !r || a->T < 2 || a->T > 16 || N2 % a->T) return 0;
+    return (N2 / r->radix[0]) % a->T == 0 ? a->T : 0;
+}
+
 // Host part of planning: the pass list and the twiddle jobs (no device work).
 int schedule_plan(fb_fft_plan_s* p, TwiddleBuilder& twb)
 {
@@ -798,6 +812,9 @@ int schedule_plan(fb_fft_plan_s* p, TwiddleBuilder& twb)
         const long long lo_off = twb.add_linear(lo_cnt, N, 1);
         const long long hi_off = twb.add_linear(hi_cnt, N, lo_cnt);
         const long long chunk = std::max(1LL, std::min(B, fourstep_chunk_bytes() / (N * 8)));
+        // composite-radix columns write their tiles whole, the rows read them
+        // as blocks
+        const long long tile = (N1 & (N1 - 1)) && (N2 & (N2 - 1)) && !tc ? fourstep_blocks(N1, N2) : 0;
         p->scratch_bytes = (size_t)(chunk * N) * sizeof(float2);
         p->group_names = {"fourstep.columns", "fourstep.rows"};
         for (long long b0 = 0; b0 < B; b0 += chunk) {
@@ -815,6 +832,12 @@ int schedule_plan(fb_fft_plan_s* p, TwiddleBuilder& twb)
             a.d.ptw_hi = reinterpret_cast<const float2*>(hi_off);
             rc = make_line_pass(r, twb, N2, nb, N1, 1, N2, N, N1, 1, N, false, true, false, false, 0, tc);
             if (rc != FB_FFT_OK) return rc;
+            if (tile) {
+                a.d.out_sk = tile, a.d.out_sc = N1;
+                a.d.out_blk = 1;
+                r.d.in_tl = ilog2ll(tile);
+                r.d.in_sn = N1, r.d.in_sc = tile;
+            }
             r.src = kBufScratch, r.src_off = 0;
             r.dst = kBufOut, r.dst_off = b0 * N;
             r.group = 1;

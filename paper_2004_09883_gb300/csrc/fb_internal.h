@@ -7,6 +7,8 @@
 
 #include <cstddef>
 
+#include "mr_config.h"
+
 namespace fbfft {
 
 constexpr int kMaxStages = 8;
@@ -92,6 +94,12 @@ struct PassDesc {
     // (0: one outer index, or 64-bit numbers).
     int T;
     unsigned tpo_mag;
+    // Composite-radix four-step rows: > 0 when the columns left the scratch in
+    // their own tiles, blocks of 2^in_tl consecutive columns of every row
+    // (value n of row k at n div 2^in_tl blocks of in_sn 2^in_tl values, then
+    // k 2^in_tl + n mod 2^in_tl).
+    int in_tl;
+    int out_blk;  // four-step columns: 1 = write such blocks
 };
 
 // Fill ns[] (product of the earlier radices) and its multiply-high
@@ -163,6 +171,7 @@ struct LineKernel {
                          // rebalances them with setmaxnreg, which needs exactly that pool)
     int lg1 = 0;         // plane pass (kind 3): log2 of the rows per plane (lg: of the row length)
     int cluster = 0;     // > 1: CTAs per thread-block cluster
+    const MrConfig* mr = nullptr;  // composite-radix pass (kind 5): its shape
 };
 // Extra shared memory of a tensor-core line pass: B^T (4 KB) + alignment.
 constexpr size_t kTcExtraSmem = 4096 + 128;

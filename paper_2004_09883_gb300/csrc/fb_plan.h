@@ -247,8 +247,9 @@ int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long
     p.kind = 5;
     p.io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
     if (L < 2 || L > FB_FFT_MAX_SMEM_LEN) return FB_FFT_ERR_UNSUPPORTED_SIZE;
-    const MrConfig c = mr_config((int)L, p.io);
-    if (c.n < 2 || !line_kernel_mr(true, (int)L, p.io).fn) return FB_FFT_ERR_UNSUPPORTED_SIZE;
+    const LineKernel k = line_kernel_mr(true, (int)L, p.io);
+    if (!k.fn || !k.mr) return FB_FFT_ERR_UNSUPPORTED_SIZE;
+    const MrConfig& c = *k.mr;
     d.L = (int)L;
     d.nst = c.n;
     for (int s = 0; s < c.n; ++s) d.radix[s] = c.radix[s];
@@ -272,12 +273,19 @@ int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long
     d.out_tfast = out_tfast ? 1 : 0;
     d.ptw = ptw ? 1 : 0;
     d.scale = 1.0f;
-    d.box_rows = 1;
+    // strided sides move as T x box_rows boxes (even strides, rows of 16 bytes
+    // and more, boxes 128-byte aligned in shared memory)
+    int br = 0;
+    for (int b = 256; b >= 1 && !br; --b)
+        if (L % b == 0 && (b == L || (b * T * 8) % 128 == 0)) br = b;
+    const bool in_ok = !in_tfast || (T % 2 == 0 && in_sn % 2 == 0 && (O == 1 || in_so % 2 == 0));
+    const bool out_ok = !out_tfast || (T % 2 == 0 && out_sk % 2 == 0 && (O == 1 || out_so % 2 == 0));
+    p.async_ok = c.in_place && br > 0 && in_ok && out_ok && C < (1LL << 31) && O < (1LL << 31);
+    d.box_rows = br > 0 ? br : 1;
     d.tpo_mag = (d.tiles_per_o > 1 && d.ntiles < (1LL << 32))
                     ? (unsigned)(((1ULL << 32) + d.tiles_per_o - 1) / d.tiles_per_o) : 0u;
-    p.smem = (size_t)(c.buf[0] + c.buf[1] + c.ptw) * sizeof(float2);
+    p.smem = 256 + (size_t)(c.buf[0] + c.buf[1] + c.ptw) * sizeof(float2);
     if (p.smem > kMaxSmemBytes) return FB_FFT_ERR_UNSUPPORTED_SIZE;
-    p.async_ok = false;
     p.grid = std::min(d.ntiles, 0x7fffffffLL);  // one tile per CTA
     return FB_FFT_OK;
 }
@@ -295,8 +303,8 @@ int make_line_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long lo
                    int max_lines = 0, bool tc = false, bool per_kernel = false)
 {
     const bool pow2_len = (L & (L - 1)) == 0;
-    // lengths with a factor 3 or 5: the composite-radix kernel (66.6 against
-    // 148.4 us on 1000-point lines x 20001, 161 against 694 us on a 120 x 150 x
+    // lengths with a factor 3 or 5: the composite-radix kernel (62.6 against
+    // 148.4 us on 1000-point lines x 20001, 146 against 694 us on a 120 x 150 x
     // 144 x 4 volume forward and back); per_kernel keeps the offset-table kernels
     if (!pow2_len && !per_kernel)
         return make_mr_pass(p, twb, L, O, C, in_sn, in_sc, in_so, out_sk, out_sc, out_so, in_tfast, out_tfast, ptw);
@@ -453,7 +461,7 @@ inline size_t line_args(LineArgs& args, const PassPlan& q, const float2* in, flo
         if (d.in_tfast && !d.off_in &&
             encode_view(&args.tm_in, d.in, d.C, d.L, O, d.in_sn, d.in_so, 1 << d.logT, d.box_rows) != 0)
             d.async_io = 0;
-        if (d.out_tfast && !d.off_out &&
+        if (d.out_tfast && !d.off_out && !d.out_blk &&
             encode_view(&args.tm_out, d.out, d.C, d.L, O, d.out_sk, d.out_so, 1 << d.logT, d.box_rows) != 0)
             d.async_io = 0;
     }

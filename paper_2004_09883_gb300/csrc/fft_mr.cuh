@@ -5,20 +5,24 @@
 // One CTA takes one tile of T lines.  The first stage's threads load their
 // butterflies straight from global memory, the stages exchange through one or
 // two shared-memory buffers, the last stage stores to global memory (with the
-// four-step twiddle and the 1/N scale).  There is no landing buffer and no
-// copy-engine traffic, so any alignment and stride takes the same path, and
-// several small CTAs per SM overlap one another's loads, stages and stores.
+// four-step twiddle and the 1/N scale): any alignment and stride takes the same
+// path, and several small CTAs per SM overlap one another's loads, stages and
+// stores.  Strided tiles with rows of 4 or 8 values (MrConfig::in_place) move by
+// TMA instead where strides and bases allow it, and all their stages work in the
+// one buffer they land in.
 //
 // What bounds it: instruction issue first (the kernels before it spent 160-200
 // thread instructions per value on four or five small run-time radices; these
-// spend 50-60), then the memory system: 1000-point lines x 20001 148.4 -> 66.6
-// us (4.8 TB/s, 0.71 of the copy rate), the passes of a 120 x 150 x 144 x 4
-// volume 103-127 -> 26-32 us each (5.2-6.3 TB/s).  Large radices cut the shared-
-// memory round trips and the twiddle multiplies to one or two per value; a
-// run-time-strided form of the same stages needed 75 instructions and 96
-// registers (83 us on the 1000-point lines), which is why the length is a
-// template parameter.  Power-of-two lengths stay on fft_p2.cuh, whose copy-engine
-// tiles measured faster there (4096 x 16384 173 against 224 us).
+// spend 40-60), then the memory system: 1000-point lines x 20001 148.4 -> 62.6
+// us (5.1 TB/s, 0.75 of the copy rate), the six passes of a 120 x 150 x 144 x 4
+// volume 694 -> 146 us (6.2-6.7 TB/s a pass).  Large radices cut the shared-memory
+// round trips and the twiddle multiplies to one or two per value; a run-time-
+// strided form of the same stages needed 75 instructions and 96 registers (83 us
+// on the 1000-point lines), which is why the length is a template parameter.
+// The narrow strided tiles are bound by latency and the load/store path:
+// 10^6 points x 16 266 -> 134 us.  Power-of-two lengths stay on fft_p2.cuh, whose
+// warp-specialised tiles measured faster there (4096 x 16384 173 against 201 us,
+// 2^20 x 32 209 against 243-269, 2048 x 2048 71 against 80).
 #pragma once
 
 #include "fft_device.cuh"
@@ -175,8 +179,9 @@ struct Mr {
     static_assert(c.n >= 2, "no schedule");
 };
 
-// Stage S of the tile whose first line starts at gin / gout.
-template <bool FWD, int L, int IO, int S>
+// Stage S of the tile whose first line starts at gin / gout.  COPIED: the strided
+// sides of the tile are in buf0 (dense, [position][line]), moved by TMA.
+template <bool FWD, int L, int IO, bool COPIED, int S>
 __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, float2* gout, float2* buf0,
                                          float2* buf1, float2* ptw, int Tv, int c0, unsigned long long pol)
 {
@@ -185,16 +190,14 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
     constexpr bool IN_T = Mr<L, IO>::IN_T, OUT_T = Mr<L, IO>::OUT_T, tfast = first ? IN_T : OUT_T;
     constexpr int R = C.radix[S], LR = L / R, Ns = C.ns[S], TH = C.threads;
     constexpr int NB = C.T * LR, Q = (NB + TH - 1) / TH;  // butterflies of a full tile, rounds
-    constexpr int Q1 = first && Q * R <= (C.regs - 32) / 2 ? Q : 1;  // rounds whose loads go out together
-    const float2* rd = (S & 1) ? buf0 : buf1;
-    float2* wr = (S & 1) ? buf1 : buf0;
+    constexpr bool land = first && IN_T && COPIED, back = last && OUT_T && COPIED;
+    // rounds whose loads go out together: all of a stage's where it writes the
+    // buffer it reads
+    constexpr bool shared = C.in_place && (first ? land : (!last || back));
+    constexpr int Q1 = shared || (first && Q * R <= (C.regs - 28) / 2) ? Q : 1;
+    const float2* rd = (S & 1) || C.in_place ? buf0 : buf1;
+    float2* wr = (S & 1) && !C.in_place ? buf1 : buf0;
     const float2* twb = d.tw + (first ? 0 : d.twoff[S]);
-    if constexpr (first && IO == 3) {  // the tile's four-step factors: last stage's r, line t
-        constexpr int RL = C.radix[C.n - 1];
-        for (int e = threadIdx.x; e < RL * C.T; e += TH)
-            if (e % C.T < Tv)  // c < C: the product stays below N
-                ptw[e] = mr_ptw(d, (unsigned)(c0 + e % C.T) * (unsigned)(e / C.T * (L / RL)));
-    }
     if constexpr (!first) __syncthreads();
 #pragma unroll
     for (int q0 = 0; q0 < Q; q0 += Q1) {
@@ -206,26 +209,54 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
             const int b = threadIdx.x + (q0 + u) * TH;
             t[u] = tfast ? b % C.T : b / LR;
             j[u] = tfast ? b / C.T : b % LR;
+            if constexpr (first && IO == 2) {
+                // rows in column-tile blocks of 2^in_tl values of every row:
+                // consecutive threads on a block's consecutive rows
+                if (d.in_tl) {
+                    t[u] = (b >> d.in_tl) % C.T;
+                    j[u] = (b >> d.in_tl) / C.T << d.in_tl | (b & ((1 << d.in_tl) - 1));
+                }
+            }
             ok[u] = ((q0 + u + 1) * TH <= NB || b < NB) && t[u] < Tv;
+            if ((shared || Q1 > 1) && !ok[u]) {
+                // defined on every path (loaded and used under one condition,
+                // which the register allocator cannot prove)
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[u][r] = make_float2(0.f, 0.f);
+            }
             if (!ok[u]) continue;
-            if constexpr (first) {
+            if constexpr (land) {
+                const float2* p = buf0 + b;  // (j + r LR) T + t, b = j T + t
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[u][r] = p[r * LR * C.T];
+            } else if constexpr (first) {
                 const float2* p = IN_T ? gin + (long long)j[u] * d.in_sn + t[u] : gin + t[u] * L + j[u];
-                const long long step = IN_T ? LR * d.in_sn : LR;
+                long long step = IN_T ? LR * d.in_sn : LR;
+                if constexpr (IO == 2) {
+                    if (d.in_tl) {
+                        const int lo = j[u] & ((1 << d.in_tl) - 1);
+                        p = gin + (long long)(j[u] - lo) * d.in_sn + (t[u] << d.in_tl) + lo;
+                        step = LR * d.in_sn;
+                    }
+                }
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u][r] = mr_ldg(p + r * step, pol);
             } else {
                 constexpr int step = LR + LR / Ns * C.pad[S];
                 const float2* p = rd + t[u] * C.row[S] + j[u] + j[u] / Ns * C.pad[S];
-                const float2* w = twb + j[u] % Ns;
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u][r] = p[r * step];
-#pragma unroll
-                for (int r = 1; r < R; ++r) v[u][r] = twmul<FWD>(v[u][r], __ldg(w + (r - 1) * Ns));
             }
         }
+        if constexpr (shared) __syncthreads();  // every value of the buffer has been read
 #pragma unroll
         for (int u = 0; u < Q1; ++u) {
             if (!ok[u]) continue;
+            if constexpr (!first) {
+                const float2* w = twb + j[u] % Ns;
+#pragma unroll
+                for (int r = 1; r < R; ++r) v[u][r] = twmul<FWD>(v[u][r], __ldg(w + (r - 1) * Ns));
+            }
             mr_dft<R, FWD>(v[u]);
             if constexpr (!last) {
                 constexpr int row = C.row[S + 1], blk = Ns * R + C.pad[S + 1];
@@ -237,11 +268,13 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
                 float2* p = OUT_T ? gout + (long long)j[u] * d.out_sk + t[u] : gout + t[u] * L + j[u];
                 const long long step = OUT_T ? Ns * d.out_sk : Ns;
                 if constexpr (IO == 3) {
-                    // exp(-2 pi i c (j + r Ns) / N) = exp(-2 pi i c j / N), one table
-                    // product per butterfly, times exp(-2 pi i c r Ns / N) from the
-                    // tile's own table of R values per line
-                    const float2 w = mr_ptw(d, (unsigned)(c0 + t[u]) * (unsigned)j[u]);
+                    // exp(-2 pi i c (j + r Ns) / N): products of the tile's own factors
+                    // (one gather per tile entry instead of two per butterfly from
+                    // tables of N, which were a quarter of this pass's L1 accesses)
+                    constexpr int R0 = C.radix[0];
                     const float2* p4 = ptw + t[u];
+                    float2 w = p4[C.ptw_a + j[u] % R0 * C.T];
+                    if constexpr (C.n > 2) w = cmul(w, p4[C.ptw_b + j[u] / R0 * C.T]);
                     v[u][0] = twmul<FWD>(v[u][0], w);
 #pragma unroll
                     for (int r = 1; r < R; ++r) v[u][r] = twmul<FWD>(v[u][r], cmul(w, p4[r * C.T]));
@@ -252,25 +285,66 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
                         for (int r = 0; r < R; ++r) v[u][r] = d.scale * v[u][r];
                     }
                 }
+                if constexpr (back) {
+                    const int b = threadIdx.x + (q0 + u) * TH;
 #pragma unroll
-                for (int r = 0; r < R; ++r) mr_stg(p + r * step, v[u][r], pol);
+                    for (int r = 0; r < R; ++r) buf0[b + r * Ns * C.T] = v[u][r];
+                } else {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) mr_stg(p + r * step, v[u][r], pol);
+                }
             }
         }
     }
+    if constexpr (first && IO == 3) {  // the tile's four-step factors, behind the stage so that its loads go out first
+        constexpr int RL = C.radix[C.n - 1], R0 = C.radix[0];
+        for (int e = threadIdx.x; e < C.ptw; e += TH) {
+            const int i = e / C.T, t = e % C.T;
+            const int m = i < RL ? i * (L / RL) : (i < RL + R0 ? i - RL : (i - RL - R0) * R0);
+            if (t < Tv) ptw[e] = mr_ptw(d, (unsigned)(c0 + t) * (unsigned)m);  // c < C: the product stays below N
+        }
+    }
+}
+
+template <bool FWD, int L, int IO, bool COPIED>
+__device__ __forceinline__ void mr_tile(const PassDesc& d, const float2* gin, float2* gout, float2* buf0,
+                                        float2* buf1, float2* ptw, int Tv, int c0, unsigned long long pin,
+                                        unsigned long long pout)
+{
+    constexpr int n = Mr<L, IO>::c.n;
+    mr_stage<FWD, L, IO, COPIED, 0>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pin);
+    mr_stage<FWD, L, IO, COPIED, 1>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
+    if constexpr (n > 2) mr_stage<FWD, L, IO, COPIED, 2>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
+    if constexpr (n > 3) mr_stage<FWD, L, IO, COPIED, 3>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
 }
 
 template <bool FWD, int L, int IO>
 __global__ void __maxnreg__((Mr<L, IO>::c.regs)) k_fft_mr(const __grid_constant__ LineArgs a)
 {
-    extern __shared__ __align__(16) unsigned char mr_smem[];
+    extern __shared__ __align__(128) unsigned char mr_smem_dyn[];
     constexpr MrConfig C = Mr<L, IO>::c;
+    constexpr bool IN_T = Mr<L, IO>::IN_T, OUT_T = Mr<L, IO>::OUT_T;
     const PassDesc& d = a.d;
-    float2* buf0 = reinterpret_cast<float2*>(mr_smem);
+    // 128 bytes for the barrier, then the buffers, 128-byte aligned for the copies
+    unsigned char* mr_smem = mr_smem_dyn + ((128u - (smem_u32(mr_smem_dyn) & 127u)) & 127u);
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(mr_smem);
+    float2* buf0 = reinterpret_cast<float2*>(mr_smem + 128);
     float2* buf1 = buf0 + C.buf[0];
     float2* ptw = buf1 + C.buf[1];
+    const bool copied = C.in_place && d.async_io != 0;
+    if constexpr (IN_T) {
+        if (copied) {
+            if (threadIdx.x == 0) {
+                mbar_init(bar, 1);
+                fence_mbar_init();
+            }
+            __syncthreads();
+        }
+    }
     pdl_start();
     const unsigned long long pin = d.evict_first ? l2_evict_first_policy() : l2_evict_normal_policy();
     const unsigned long long pout = d.evict_last ? l2_evict_last_policy() : l2_evict_normal_policy();
+    unsigned phase = 0;
     for (long long tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) {
         // tile = o tiles_per_o + rest: below 2^32 by the reciprocal
         // ceil(2^32 / tiles_per_o), which is at most one too high
@@ -285,11 +359,45 @@ __global__ void __maxnreg__((Mr<L, IO>::c.regs)) k_fft_mr(const __grid_constant_
         const int Tv = d.C - c0 < d.T ? (int)(d.C - c0) : d.T;
         const float2* gin = d.in + o * d.in_so + c0 * d.in_sc;
         float2* gout = d.out + o * d.out_so + c0 * d.out_sc;
-        if (tile != blockIdx.x) __syncthreads();  // the last tile's exchange buffers are free
-        mr_stage<FWD, L, IO, 0>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pin);
-        mr_stage<FWD, L, IO, 1>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pout);
-        if constexpr (C.n > 2) mr_stage<FWD, L, IO, 2>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pout);
-        if constexpr (C.n > 3) mr_stage<FWD, L, IO, 3>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pout);
+        if (tile != blockIdx.x) __syncthreads();  // the last tile's buffers are free (copies: read, below)
+        if constexpr (IN_T) {
+            if (copied) {
+                if (threadIdx.x == 0) {
+                    mbar_arrive_expect_tx(bar, (unsigned)(C.T * L) * 8u + d.debug_extra_tx);
+                    for (int n0 = 0; n0 < L; n0 += d.box_rows)
+                        tma_load_3d(buf0 + n0 * C.T, &a.tm_in, (int)c0, n0, (int)o, bar, d.err, true, pin);
+                }
+                const bool bad = !mbar_wait_bounded(bar, phase);
+                phase ^= 1u;
+                if (__syncthreads_or(bad)) {
+                    if (threadIdx.x == 0) atomicExch(d.err, 1);
+                    return;
+                }
+            }
+        }
+        if (C.in_place && copied)
+            mr_tile<FWD, L, IO, C.in_place>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pin, pout);
+        else
+            mr_tile<FWD, L, IO, false>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pin, pout);
+        if constexpr (OUT_T) {
+            if (copied) {
+                fence_proxy_async();  // the tile -> visible to the copy engine
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    if (d.out_blk) {  // column-tile blocks: the tile as it lies here
+                        bulk_store_1d(gout, buf0, (unsigned)(C.T * L) * 8u, d.err, true, pout);
+                    } else {
+                        for (int k0 = 0; k0 < L; k0 += d.box_rows)
+                            tma_store_3d(&a.tm_out, (int)c0, k0, (int)o, buf0 + k0 * C.T, d.err, true, pout);
+                    }
+                    bulk_commit();
+                    bulk_wait_read_all();  // before the buffer is written again or the CTA leaves
+                }
+            }
+        }
+    }
+    if constexpr (OUT_T) {
+        if (copied && threadIdx.x == 0) bulk_wait_all();
     }
 }
 
@@ -298,6 +406,7 @@ LineKernel mr_entry()
 {
     LineKernel k = make_entry<Mr<L, IO>::c.threads>(k_fft_mr<FWD, L, IO>, FWD, L, IO);
     k.kind = 5;
+    k.mr = &Mr<L, IO>::c;
     return k;
 }
 

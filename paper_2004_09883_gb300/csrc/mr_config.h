@@ -45,11 +45,12 @@ constexpr void mr_search(int n, int from, int left, MrSchedule cur, MrSchedule& 
 // more of them a thread has in flight the better).  A length of one radix ends
 // with a radix-1 copy, and on contiguous lines starts with one too, so that
 // global accesses stay on consecutive values.
-constexpr MrSchedule mr_schedule(int L, bool contiguous)
+constexpr MrSchedule mr_schedule(int L, bool contiguous, int max_radix = 25)
 {
     MrSchedule best{};
-    int sum = 0;
-    for (int n = 1; n <= kMrMaxStages && best.n == 0; ++n) mr_search(L, 0, n, MrSchedule{}, best, sum);
+    int sum = 0, from = 0;
+    while (kMrRadices[from] > max_radix) ++from;
+    for (int n = 1; n <= kMrMaxStages && best.n == 0; ++n) mr_search(L, from, n, MrSchedule{}, best, sum);
     if (best.n != 1) return best;
     const int r = best.radix[0];
     MrSchedule s{};
@@ -73,8 +74,14 @@ struct MrConfig {
     // reader's index both split along them.
     int pad[kMrMaxStages];
     int row[kMrMaxStages];
-    int buf[2];                 // values of the two exchange buffers (exchange s uses s - 1 & 1)
-    int ptw;                    // values of the tile's four-step factors, behind them (io 3)
+    int buf[2];                 // values of the two exchange buffers (exchange s uses s - 1 & 1);
+                                // buf[1] = 0: every exchange uses buffer 0 (see in_place)
+    bool in_place;              // every stage reads all its values before any is written
+    // The tile's four-step factors exp(-2 pi i c m / N) of its lines c, behind
+    // the buffers (io 3): m = r ns[n-1] for the outputs of a last-stage
+    // butterfly, then the two parts of its position j = a + radix[0] b: m = a,
+    // m = radix[0] b (three stages and more).  T values each.
+    int ptw_a, ptw_b, ptw;      // where m = a and m = radix[0] b start, and all of them
 };
 
 constexpr bool mr_in_t(int io) { return io == 1 || io == 3; }
@@ -85,16 +92,17 @@ constexpr bool mr_out_t(int io) { return io != 0; }
 constexpr bool mr_tfast(int io, int s) { return s == 0 ? mr_in_t(io) : mr_out_t(io); }
 
 // Shared-memory wavefronts (8-byte words, half a warp at a time, 16 banks) of
-// the first 64 threads writing and reading exchange e with rows of `row`.
+// the first 32 threads writing and reading exchange e with rows of `row`.
 constexpr int mr_wavefronts(const MrConfig& c, int e, int row)
 {
     int total = 0;
     for (int side = 0; side < 2; ++side) {
-        const int s = e - 1 + side, LR = c.L / c.radix[s], nb = c.T * LR < 64 ? c.T * LR : 64;
+        const int s = e - 1 + side, LR = c.L / c.radix[s], nb = c.T * LR < 32 ? c.T * LR : 32;
         for (int h = 0; h < nb; h += 16) {
             int count[16] = {}, worst = 0;
             for (int b = h; b < h + 16 && b < nb; ++b) {
-                const int t = mr_tfast(c.io, s) ? b % c.T : b / LR, j = mr_tfast(c.io, s) ? b / c.T : b % LR;
+                int t = mr_tfast(c.io, s) ? b % c.T : b / LR, j = mr_tfast(c.io, s) ? b / c.T : b % LR;
+                if (c.io == 2 && s == 0) t = b / 4 % c.T, j = b / (4 * c.T) * 4 + b % 4;  // column-tile blocks
                 const int at = side ? t * row + j + j / c.ns[e] * c.pad[e]
                                     : t * row + j / c.ns[e - 1] * (c.ns[e] + c.pad[e]) + j % c.ns[e - 1];
                 const int n = ++count[at & 15];
@@ -105,6 +113,56 @@ constexpr int mr_wavefronts(const MrConfig& c, int e, int row)
     }
     return total;
 }
+
+// Place the exchange buffers of a shape whose L, io, n, radix, ns and T are set.
+constexpr void mr_place(MrConfig& c)
+{
+    const int L = c.L;
+    for (int e = 1; e < c.n; ++e) {
+        // Writer: groups of Nw consecutive values, the next group R Nw + pad
+        // further on; half a warp covers consecutive groups without a bank
+        // met twice when that stride is Nw mod 16 (8-byte words), or, for
+        // Nw = 1, odd.  No pad where that is no better (tiles of 8 lines and
+        // more spread a half-warp over their rows).
+        const int Nw = c.ns[e - 1], R = c.radix[e - 1], blk = c.ns[e];
+        int want = Nw == 1 ? (R % 2 == 0) : ((Nw - Nw * R) % 16 + 16) % 16;
+        if (Nw > 1 && want * 8 > blk) want = 0;
+        int row = L, best = 1 << 30, best_pad = 0;
+        for (int k = 0; k < (want ? 2 : 1); ++k) {
+            c.pad[e] = k ? want : 0;
+            const int ext = L + (L / blk - 1) * c.pad[e];
+            // The row stride: lines of 32 butterflies and more side by side
+            // hardly meet, any will do; stages across the lines on both sides
+            // want rows an odd multiple of H = 16 / T apart (half a warp holds H
+            // positions of T lines); else the one of 16 with the fewest conflicts.
+            const bool tw = mr_tfast(c.io, e - 1), tr = mr_tfast(c.io, e);
+            const int H = c.T < 16 ? 16 / c.T : 1;
+            int x0 = 0, x1 = 1;
+            if (tw && tr)
+                for (x0 = 0; (ext + x0) % (2 * H) != H;) ++x0;
+            else if (c.T > 1 && (tw || tr || L / R < 32 || L / c.radix[e] < 32))
+                x1 = 16;
+            if (tw && tr) x1 = x0 + 1;
+            for (int x = x0; x < x1; ++x) {
+                const int cost = mr_wavefronts(c, e, ext + x);
+                if (cost < best) best = cost, best_pad = c.pad[e], row = ext + x;
+            }
+        }
+        c.pad[e] = best_pad;
+        c.row[e] = row;
+        int& b = c.buf[c.in_place ? 0 : (e - 1) & 1];
+        b = c.T * row > b ? c.T * row : b;
+    }
+    if (c.in_place && c.buf[0] < L * c.T) c.buf[0] = L * c.T;  // the tile itself, as copied in and out
+    c.buf[0] = (c.buf[0] + 1) & ~1;
+    c.ptw_a = c.T * c.radix[c.n - 1];
+    c.ptw_b = c.ptw_a + c.T * c.radix[0];
+    c.ptw = c.io != 3 ? 0 : c.ptw_b + (c.n > 2 ? c.T * (c.ns[c.n - 1] / c.radix[0]) : 0);
+}
+
+// Registers a thread of a CTA can have: each quarter of an SM holds 16384, and
+// the CTA's warps are dealt out to the quarters one by one.
+constexpr int mr_reg_cap(int threads) { return 16384 / (32 * ((threads + 127) / 128)) / 8 * 8; }
 
 constexpr MrConfig mr_config(int L, int io)
 {
@@ -137,41 +195,51 @@ constexpr MrConfig mr_config(int L, int io)
         }
     } else {
         // A strided side moves rows of T values: 16 (128 bytes) up to 256
-        // points, 8 up to 512, 4 (one 32-byte sector) up to 2048, then 2.
+        // points, 8 up to 540, 4 (one 32-byte sector) up to 2048, then 2.
         c.T = L <= 256 ? 16 : (L <= 540 ? 8 : (L <= 2048 ? 4 : 2));
     }
-    int nbmax = 1;
-    for (int i = 0; i < c.n; ++i) {
-        const int nb = c.T * (L / c.radix[i]);
-        nbmax = nb > nbmax ? nb : nbmax;
-    }
-    const int rounds = (nbmax + 255) / 256;
-    c.threads = ((nbmax + rounds - 1) / rounds + 31) / 32 * 32;
-    c.regs = rmax <= 10 ? 64 : (rmax <= 16 ? 80 : (rmax <= 20 ? 96 : 112));
-    for (int e = 1; e < c.n; ++e) {
-        // Writer: groups of Nw consecutive values, the next group R Nw + pad
-        // further on; half a warp covers consecutive groups without a bank
-        // met twice when that stride is Nw mod 16 (8-byte words), or, for
-        // Nw = 1, odd.  Tiles of 16 lines spread a half-warp over their rows
-        // instead and need no pad.  The row stride is the one of 16 with the
-        // fewest conflicts.
-        const int Nw = c.ns[e - 1], R = c.radix[e - 1], blk = c.ns[e];
-        const bool by_rows = c.T >= 16 && mr_tfast(io, e - 1) && mr_tfast(io, e);
-        int pad = by_rows ? 0 : (Nw == 1 ? (R % 2 == 0) : ((Nw - Nw * R) % 16 + 16) % 16);
-        if (Nw > 1 && pad * 8 > blk) pad = 0;
-        c.pad[e] = pad;
-        const int ext = L + (L / blk - 1) * pad;
-        int row = ext, best = 1 << 30;
-        for (int x = 0; x < (c.T > 1 ? 16 : 1); ++x) {
-            const int cost = mr_wavefronts(c, e, ext + x);
-            if (cost < best) best = cost, row = ext + x;
+    c.regs = rmax <= 10 ? 48 : (rmax <= 12 ? 56 : (rmax <= 16 ? 64 : (rmax <= 20 ? 80 : 96)));
+    if (io == 0 || c.n == 2 || c.T >= 16 || L > 1024) {
+        // Contiguous lines, and strided tiles but for those below: straight
+        // between global memory and registers, small CTAs, several per SM -- the
+        // fewest rounds of 320 threads (strided: 512, or 256 for the long lines'
+        // large tiles), then the fewest threads.
+        int rounds = 1 << 30;
+        for (int th = 64; th <= (io == 0 ? 320 : (L > 1024 ? 256 : 512)); th += 32) {
+            int all = 0;
+            for (int i = 0; i < c.n; ++i) all += (c.T * (L / c.radix[i]) + th - 1) / th;
+            if (all < rounds) rounds = all, c.threads = th;
         }
-        c.row[e] = row;
-        int& b = c.buf[(e - 1) & 1];
-        b = c.T * row > b ? c.T * row : b;
+    } else {
+        // Strided tiles of three stages and more, rows of 4 or 8 values: the
+        // copy engine moves them, which spares the load and store path one access
+        // per 32-byte piece, and every stage works in the tile's own buffer: it
+        // reads all its values before any is written, so a thread holds `held`
+        // values at once.  One round per stage where 1024 threads reach it (two
+        // butterflies held at once spill), then the fewest threads.  10^6 points x
+        // 16: 205 -> 134 us with this and the tile's own factors below (1000 x 64
+        // grids x 80: 39.6 -> 34.1 us).  Slower this way: tiles of two stages (120 x
+        // 150 x 144 x 4: 163 against 146 us), rows of 16 (65610 points x 200, 243-
+        // point columns: 127 against 101), and lines above 1024 points, whose tile
+        // then has an SM to itself (1500 x 64 grids x 50: 45 against 39).
+        int held = 0, cost = 1 << 30;
+        for (int th = 64; th <= 1024; th += 32) {
+            int most = 0, worst = 0;
+            for (int i = 0; i < c.n; ++i) {
+                const int q = (c.T * (L / c.radix[i]) + th - 1) / th, h = q * c.radix[i];
+                const int w = q > 1 && h > 12 ? h + 8 : h;
+                most = h > most ? h : most;
+                worst = w > worst ? w : worst;
+            }
+            if ((2 * most + 28 + 7) / 8 * 8 > mr_reg_cap(th) || worst >= cost) continue;
+            cost = worst, held = most, c.threads = th;
+        }
+        c.in_place = true;
+        const int need = (2 * held + 28 + 7) / 8 * 8, cap = mr_reg_cap(c.threads);
+        c.regs = need > c.regs ? need : c.regs;
+        c.regs = c.regs < cap ? c.regs : cap;
     }
-    c.buf[0] = (c.buf[0] + 1) & ~1;
-    c.ptw = io == 3 ? c.radix[c.n - 1] * c.T : 0;
+    mr_place(c);
     return c;
 }
 

@@ -8,6 +8,7 @@
 #include <cmath>
 #include <complex>
 #include <cstdio>
+#include <utility>
 #include <vector>
 
 #include "fft_mr.cuh"
@@ -71,7 +72,9 @@ static long long run_tile(const MrConfig& c, int Tv, double* err)
     for (int st = 0; st < nst; ++st) {
         const bool first = st == 0, last = st == nst - 1;
         const bool tf = mr_tfast(c.io, st);
-        const int R = c.radix[st], LR = L / R, Ns = c.ns[st], rb = (st - 1) & 1, wb = st & 1;
+        const int R = c.radix[st], LR = L / R, Ns = c.ns[st];
+        const int rb = c.in_place ? 0 : (st - 1) & 1, wb = c.in_place ? 0 : st & 1;
+        std::vector<std::pair<long long, float2>> out;  // written once every value of the stage is read
         for (int b = 0; b < c.T * LR; ++b) {
             const int t = tf ? b % c.T : b / LR, j = tf ? b / c.T : b % LR, q = j / Ns, k = j % Ns;
             if (t >= Tv) continue;
@@ -92,15 +95,19 @@ static long long run_tile(const MrConfig& c, int Tv, double* err)
                 if (!last) {
                     const int blk = Ns * R + c.pad[st + 1];
                     const long long at = (long long)t * c.row[st + 1] + (long long)q * blk + k + (long long)r * Ns;
-                    if (at < 0 || at >= c.buf[wb] || mark[wb][at] == st + 1) { ++bad; continue; }
-                    mark[wb][at] = st + 1;
-                    buf[wb][at] = v[r];
+                    if (at < 0 || at >= c.buf[wb]) { ++bad; continue; }
+                    out.push_back({at, v[r]});
                 } else {
                     const int kk = j + r * Ns;
                     if (kk >= L || wrote[t * (size_t)L + kk]++) { ++bad; continue; }
                     y[t][kk] = v[r];
                 }
             }
+        }
+        for (auto& o : out) {
+            bad += mark[wb][o.first] == st + 1;
+            mark[wb][o.first] = st + 1;
+            buf[wb][o.first] = o.second;
         }
     }
     for (int w : wrote) bad += w != 1;
@@ -128,7 +135,7 @@ int main()
             const MrConfig c = mr_config(L, io);
             bad += c.n < 2 || c.n > kMrMaxStages;
             bad += io != 0 && (c.T & (c.T - 1)) != 0;
-            bad += c.threads > 512 || c.threads % 32 != 0 || c.threads * c.regs > 65536;
+            bad += c.threads > 1024 || c.threads % 32 != 0 || c.regs > mr_reg_cap(c.threads);
             bad += (c.buf[0] + c.buf[1]) * 8 > 227 * 1024;
             for (int Tv : {c.T, (c.T + 1) / 2, 1}) {
                 bad += run_tile<true>(c, Tv, &err);
@@ -138,5 +145,36 @@ int main()
         }
     }
     std::printf("mr_pass %lld %lld %.3e\n", cases, bad, err);
+    // rows read from column-tile blocks: every value of every row once, from
+    // where the column pass puts it (value n of row k: block n / 2^tl of N1 2^tl
+    // values, in it row k's run)
+    cases = bad = 0;
+    for (int L = 16; L <= 4096; ++L) {
+        int n = L;
+        for (int p : {2, 3, 5})
+            while (n % p == 0) n /= p;
+        if (n != 1) continue;
+        const MrConfig c = mr_config(L, 2);
+        const int R = c.radix[0], LR = L / R;
+        for (int tl = 1; tl <= 4; ++tl) {
+            if (LR % (1 << tl)) continue;
+            const long long N1 = 1000;
+            std::vector<int> seen((size_t)c.T * L, 0);
+            for (int b = 0; b < c.T * LR; ++b) {
+                const int t = (b >> tl) % c.T, j = (b >> tl) / c.T << tl | (b & ((1 << tl) - 1));
+                bad += j < 0 || j >= LR;
+                const int lo = j & ((1 << tl) - 1);
+                for (int r = 0; r < R && j < LR; ++r) {
+                    const int v = j + r * LR;
+                    bad += (j - lo) * N1 + (t << tl) + lo + (long long)r * LR * N1 !=
+                           (v >> tl) * (N1 << tl) + (t << tl) + (v & ((1 << tl) - 1));
+                    ++seen[(size_t)t * L + v];
+                }
+            }
+            for (int x : seen) bad += x != 1;
+            ++cases;
+        }
+    }
+    std::printf("row_blocks %lld %lld 0\n", cases, bad);
     return 0;
 }

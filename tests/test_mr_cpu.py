@@ -24,3 +24,5 @@ def test_composite_radix_pass_on_the_host(tmp_path):
     assert out[0] == "mr_pass" and int(out[1]) > 1500
     assert int(out[2]) == 0
     assert float(out[3]) < 2e-6
+    # four-step rows reading the columns' own tiles
+    assert out[4] == "row_blocks" and int(out[5]) > 100 and int(out[6]) == 0
