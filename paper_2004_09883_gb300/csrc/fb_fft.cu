@@ -236,7 +236,6 @@ struct fb_fft_plan_s {
         std::vector<int> jobs;   // pass indices
         long long tiles = 0;
         long long grid = 0;
-        int land_max = 16, work_max = 16;
         size_t smem = 0;
         PassDesc* d_jobs = nullptr;
         int* d_tiles = nullptr;
@@ -247,8 +246,9 @@ struct fb_fft_plan_s {
     // chunk's columns through device counters
     bool uneven_one = false;
     int uneven_slots = 0;                  // dependency slots: one per four-step chunk
+    long long uneven_columns = 0;          // column tiles of all chunks
     UnevenPhase uone;                      // the merged table's jobs, tiles, grid, shared memory
-    unsigned long long* d_sync = nullptr;  // [2 + uneven_slots] counters, zero between execs
+    unsigned long long* d_sync = nullptr;  // [3 + uneven_slots] counters, zero between execs
     void* d_uneven = nullptr;              // one allocation: job and tile tables, counters
     std::vector<MultiLaunch> multis;
     std::unique_ptr<MultiArgs> margs;      // launch-argument staging (copied at every launch)
@@ -324,39 +324,8 @@ bool use_uneven_engine(int count, const long long* lengths, const fb_fft_many_op
     return true;
 }
 
-// Radix schedule of a line of the one-kernel batched-uneven engine
-// (k_fft_uneven): the power-of-two part as radix-8 stages and one radix-4 or
-// radix-2 stage, then the 5s, then the 3s -- the order of kinds the kernel
-// runs its middle stages in.  The kernel has no one-stage form, so a
-// schedule of a single radix ends with a radix-1 stage (a copy).  Returns the
-// stage count.
-int uneven_factorize(long long L, int* r)
-{
-    int c = 0, a = 0;
-    long long n = L;
-    while (n % 2 == 0) n /= 2, ++a;
-    for (int i = 0; i < a / 3; ++i) r[c++] = 8;
-    if (a % 3 == 2) r[c++] = 4;
-    if (a % 3 == 1) r[c++] = 2;
-    while (n % 5 == 0) n /= 5, r[c++] = 5;
-    while (n % 3 == 0) n /= 3, r[c++] = 3;
-    while (c < 2) r[c++] = 1;
-    return c;
-}
-
-// Lines per tile of a job of L-point lines (C per outer index) on the
-// one-kernel engine: as many as fit 2048 values, a power of two, at most 32
-// where a side is strided (rows of T consecutive values), at most C rounded up.
-long long uneven_tile_lines(long long L, long long C, bool cfast)
-{
-    long long T = pow2floor(kUnevenCap / L);
-    T = std::min<long long>(T, cfast ? 32 : kUnevenThreads);
-    return std::max<long long>(1, std::min(T, pow2ceil(C)));
-}
-
 // One job of the one-kernel engine: L-point DFTs over lines (o, c), strides in
-// elements (offsets into the exec buffers are set by the caller); tiles of T
-// lines, T L <= 2048 values.
+// elements (offsets into the exec buffers are set by the caller).
 int make_uneven_pass(PassPlan& p, TwiddleBuilder& twb, long long L, long long O, long long C, long long in_sn,
                      long long in_sc, long long in_so, long long out_sk, long long out_sc, long long out_so,
                      bool in_tfast, bool out_tfast, bool ptw)
@@ -365,16 +334,29 @@ int make_uneven_pass(PassPlan& p, TwiddleBuilder& twb, long long L, long long O,
     PassDesc& d = p.d;
     if (L < 1 || L > kUnevenMaxLen || !is_smooth(L)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
     p.kind = 4;
-    p.io = -1;
+    p.io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
     p.threads = kUnevenThreads;
-    d.nst = uneven_factorize(L, d.radix);
+    MrConfig c = uneven_shape(L, C, p.io);
+    if (c.n < 2) return FB_FFT_ERR_UNSUPPORTED_SIZE;
+    mr_place(c);
+    d.nst = c.n;
+    for (int s = 0; s < c.n; ++s) d.radix[s] = c.radix[s];
     set_stage_products(d);
     const std::vector<int> off = twb.add_stages(L, d.radix, d.nst);
-    for (int s = 0; s < d.nst; ++s) d.twoff[s] = off[s];
-    const bool cfast = in_tfast || out_tfast;
-    const long long T = uneven_tile_lines(L, C, cfast);
+    for (int s = 0; s < d.nst; ++s) {
+        const int lr = (int)L / c.radix[s];
+        d.twoff[s] = off[s];
+        d.lr_mag[s] = lr > 1 ? (unsigned)(((1ULL << 32) + lr - 1) / lr) : 0u;
+        if (s == 0) continue;
+        d.xrow[s] = c.row[s];
+        d.xpad[s] = c.pad[s];
+        d.xstep[s] = lr + lr / c.ns[s] * c.pad[s];
+    }
+    d.xbuf = c.buf[0];
+    d.ptw_at = c.buf[0] + c.buf[1];
+    const long long T = c.T;
     d.L = (int)L;
-    d.LS = uneven_line_stride(L, T, cfast);
+    d.T = (int)T;
     d.logT = ilog2ll(T);
     d.in_sn = in_sn, d.in_sc = in_sc, d.in_so = in_so;
     d.out_sk = out_sk, d.out_sc = out_sc, d.out_so = out_so;
@@ -385,39 +367,26 @@ int make_uneven_pass(PassPlan& p, TwiddleBuilder& twb, long long L, long long O,
     d.out_tfast = out_tfast ? 1 : 0;
     d.ptw = ptw ? 1 : 0;
     d.scale = 1.0f;
-    d.land_row = uneven_land_row(L, T, in_tfast);
-    d.land_stride = (int)(((d.land_row ? d.land_row : L) * T + 15) & ~15LL);
     p.async_ok = false;
-    const int padded = (int)(((long long)d.LS * T + 15) & ~15LL);
-    p.smem = uneven_smem_bytes(std::max(d.land_stride, padded), padded);
+    p.smem = (size_t)(c.buf[0] + c.buf[1] + c.ptw) * sizeof(float2);
     p.grid = 0;  // launched through its phase's launch only
     return FB_FFT_OK;
 }
 
-// Issue cost of one tile in k_fft_uneven, in values handled per thread: per
-// stage, the butterfly rounds a thread runs (radix R values each) plus a
-// fixed stage overhead, plus the tile's load and store.  A tile of T lines
-// has 256 / T threads per line; the cost hardly depends on how full the tile
-// is, so lengths whose tiles stay half empty cost twice per value.
-long long uneven_tile_cost(long long L, long long T)
+// Issue cost of one tile of L-point lines with a strided side in k_fft_uneven,
+// in warp instructions: per stage of radix R, a butterfly is about 14 R + 30.
+long long uneven_tile_cost(const MrConfig& c)
 {
-    int r[kMaxStages];
-    const int nst = uneven_factorize(L, r);
-    const long long G = kUnevenThreads / T;
-    long long c = 10;
-    for (int s = 0; s < nst; ++s) {
-        const long long LR = L / r[s];
-        c += (LR + G - 1) / G * r[s] + 6;
-    }
-    return c;
+    long long cost = 300;
+    for (int s = 0; s < c.n; ++s) cost += (c.T * (c.L / c.radix[s]) + 31) / 32 * (14LL * c.radix[s] + 30);
+    return cost;
 }
 
 // The four-step split of n > 2048 on the one-kernel engine: n = n1 * n2 (the
 // column and row lengths), both at most 2048.  Among all such pairs, the one
-// whose two jobs cost the fewest tile issues per transform (above), keeping
+// whose two jobs cost the fewest instructions per transform (above), keeping
 // the strided rows at least as long as the split with the largest n1 <= sqrt(n)
-// has them (up to 8 values): on 4096 lengths in [64, 65536] this cut the
-// modelled issue cost by 7 %.
+// has them (up to 8 values).
 int split_uneven(long long n, long long* n1, long long* n2)
 {
     long long base = 0;
@@ -426,13 +395,14 @@ int split_uneven(long long n, long long* n1, long long* n2)
     if (base == 0) return FB_FFT_ERR_UNSUPPORTED_SIZE;
     auto seg = [&](long long a) {  // shorter strided row of the pair (a, n / a)
         const long long b = n / a;
-        return std::min(uneven_tile_lines(a, b, true), uneven_tile_lines(b, a, true));
+        return std::min(uneven_shape(a, b, kIoCCP).T, uneven_shape(b, a, kIoNC).T);
     };
     auto cost = [&](long long a) {
-        const long long b = n / a, ta = uneven_tile_lines(a, b, true), tb = uneven_tile_lines(b, a, true);
-        return (b + ta - 1) / ta * uneven_tile_cost(a, ta) + (a + tb - 1) / tb * uneven_tile_cost(b, tb);
+        const long long b = n / a;
+        const MrConfig ca = uneven_shape(a, b, kIoCCP), cb = uneven_shape(b, a, kIoNC);
+        return (b + ca.T - 1) / ca.T * uneven_tile_cost(ca) + (a + cb.T - 1) / cb.T * uneven_tile_cost(cb);
     };
-    const long long min_seg = std::min<long long>(8, seg(base));
+    const int min_seg = std::min(8, seg(base));
     long long best = base, best_cost = cost(base);
     for (long long a = 1; a <= kUnevenMaxLen && a <= n; ++a) {
         if (n % a || n / a > kUnevenMaxLen || seg(a) < min_seg) continue;
@@ -526,6 +496,7 @@ int schedule_uneven(fb_fft_plan_s* p, TwiddleBuilder& twb)
             r.d.dep = slot + 1;
             if (a.d.ntiles >= (1LL << 31)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
             r.d.dep_need = (int)a.d.ntiles;
+            p->uneven_columns += a.d.ntiles;
             p->passes.push_back(a);
             p->passes.push_back(r);
         }
@@ -536,19 +507,14 @@ int schedule_uneven(fb_fft_plan_s* p, TwiddleBuilder& twb)
         fb_fft_plan_s::UnevenPhase& ph = p->uphase[q.group];
         ph.jobs.push_back(i);
         ph.tiles += q.d.ntiles;
-        const int padded = (int)(((long long)q.d.LS * (1LL << q.d.logT) + 15) & ~15LL);
-        ph.land_max = std::max(ph.land_max, std::max(q.d.land_stride, padded));  // also a work buffer
-        ph.work_max = std::max(ph.work_max, padded);
+        ph.smem = std::max(ph.smem, q.smem);
     }
-    for (auto& ph : p->uphase) ph.smem = uneven_smem_bytes(ph.land_max, ph.work_max);
     fb_fft_plan_s::UnevenPhase& one = p->uone;
     for (const fb_fft_plan_s::UnevenPhase& ph : p->uphase) {
         one.jobs.insert(one.jobs.end(), ph.jobs.begin(), ph.jobs.end());
         one.tiles += ph.tiles;
-        one.land_max = std::max(one.land_max, ph.land_max);
-        one.work_max = std::max(one.work_max, ph.work_max);
+        one.smem = std::max(one.smem, ph.smem);
     }
-    one.smem = uneven_smem_bytes(one.land_max, one.work_max);
     p->scratch_bytes = (size_t)scratch_need * sizeof(float2);
     p->tw_elems = std::max(2LL, twb.total);
     return FB_FFT_OK;
@@ -1031,7 +997,7 @@ int build_plan(fb_fft_plan_s* p)
             }
             const size_t jb = jobs.size() * sizeof(PassDesc), tb = tiles.size() * sizeof(int);
             const size_t sb_at = (jb + tb + 15) & ~(size_t)15;
-            const int nsync = 2 + p->uneven_slots;
+            const int nsync = 3 + p->uneven_slots;
             const size_t sb = (size_t)nsync * sizeof(unsigned long long);
             if (cudaMalloc(&p->d_uneven, sb_at + sb) != cudaSuccess) {
                 cudaGetLastError();
@@ -1240,11 +1206,10 @@ int launch_uneven(fb_fft_plan_s* p, cudaStream_t stream, const float2* in, float
         a.out = out;
         a.scratch = p->scratch;
         a.njobs = (int)u.jobs.size();
-        a.land_max = u.land_max;
-        a.work_max = u.work_max;
         a.scale_on = (!fwd && (p->flags & FB_FFT_SCALE_INV_N)) ? 1 : 0;
         a.sync = p->d_sync;
-        a.nsync = 2 + p->uneven_slots;
+        a.nsync = 3 + p->uneven_slots;
+        a.columns = (int)p->uneven_columns;
         a.dep_extra = p->debug_timeout ? (1 << 30) : 0;
         cudaEvent_t e1 = nullptr;
         if (p->profiling) {
@@ -1627,9 +1592,7 @@ int recipe_create(BatchRecipe** out, int rank, const long long* dims, long long 
         j.src = q.src == kBufIn ? 0 : (q.src == kBufOut ? 1 : 2);
         j.dst = q.dst == kBufOut ? 1 : 2;
         j.last = q.last;
-        const int padded = (int)(((long long)q.d.LS * (1LL << q.d.logT) + 15) & ~15LL);
-        j.land = std::max(q.d.land_stride, padded);  // also serves as a work buffer
-        j.work = padded;
+        j.smem = q.smem;
         r->jobs.push_back(j);
         r->phases = std::max(r->phases, q.group + 1);
         r->tiles += q.d.ntiles;
@@ -1672,11 +1635,10 @@ int uneven_resident(bool forward, size_t smem, bool inl, long long* cap)
 }
 
 int batch_launch(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
-                 int land_max, int work_max, cudaStream_t stream)
+                 size_t smem, cudaStream_t stream)
 {
     if (njobs <= 0 || tiles <= 0) return FB_FFT_OK;
     if (tiles >= (1LL << 31)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
-    const size_t smem = uneven_smem_bytes(land_max, work_max);
     long long cap = 0;
     int rc = uneven_resident(forward, smem, false, &cap);
     if (rc != FB_FFT_OK) return rc;
@@ -1687,8 +1649,6 @@ int batch_launch(bool forward, const PassDesc* jobs, const int* tile_start, int 
     a.out = nullptr;
     a.scratch = nullptr;
     a.njobs = njobs;
-    a.land_max = land_max;
-    a.work_max = work_max;
     a.scale_on = 1;  // each job's apply_scale says whether it scales
     const cudaError_t e = uneven_launch(forward, a, std::min(tiles, cap), smem, stream);
     if (e != cudaSuccess) return cuda_fail(e, "k_fft_uneven (server batch)");
@@ -1697,20 +1657,17 @@ int batch_launch(bool forward, const PassDesc* jobs, const int* tile_start, int 
 }
 
 int batch_launch_inline(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
-                        int land_max, int work_max, cudaStream_t stream)
+                        size_t smem, cudaStream_t stream)
 {
     if (njobs <= 0 || tiles <= 0) return FB_FFT_OK;
     if (njobs > kUnevenInlineJobs) return FB_FFT_ERR_INVALID_ARG;
     if (tiles >= (1LL << 31)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
-    const size_t smem = uneven_smem_bytes(land_max, work_max);
     long long cap = 0;
     int rc = uneven_resident(forward, smem, true, &cap);
     if (rc != FB_FFT_OK) return rc;
     UnevenInlineArgs p;
     std::memset(&p, 0, sizeof(p));
     p.a.njobs = njobs;
-    p.a.land_max = land_max;
-    p.a.work_max = work_max;
     p.a.scale_on = 1;
     std::memcpy(p.jobs, jobs, (size_t)njobs * sizeof(PassDesc));
     std::memcpy(p.tile_start, tile_start, (size_t)(njobs + 1) * sizeof(int));

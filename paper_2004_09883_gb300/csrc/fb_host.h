@@ -33,7 +33,7 @@ struct BatchJob {
     int phase;        // launch it runs in: jobs of phase k + 1 read what phase k wrote
     int src, dst;     // 0 the request's input, 1 its output, 2 its scratch
     bool last;        // the job that finishes the transform (takes the 1/N scale)
-    int land, work;   // landing / work buffer elements its tiles need
+    size_t smem;      // shared memory its tiles need (bytes)
 };
 // Every job of one request shape (rank, dims, batch): up to three phases
 // (one per axis of a 2-D / 3-D shape; columns then rows of a 1-D four-step
@@ -55,11 +55,11 @@ void recipe_free(BatchRecipe* r);
 // One launch of k_fft_uneven over the job and tile-prefix tables in device
 // memory (njobs jobs, `tiles` tiles in all); the launch counter counts it.
 int batch_launch(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
-                 int land_max, int work_max, cudaStream_t stream);
+                 size_t smem, cudaStream_t stream);
 // The same launch with the tables (host memory, at most 16 jobs) copied
 // into the kernel parameter: nothing to copy to the device beforehand.
 int batch_launch_inline(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
-                        int land_max, int work_max, cudaStream_t stream);
+                        size_t smem, cudaStream_t stream);
 // Record a failed CUDA call for fb_fft_last_error and map it to a status.
 int fail(cudaError_t e, const char* what);
 

@@ -78,10 +78,6 @@ struct PassDesc {
     // the pointer fields are the addresses themselves.
     int in_buf;
     int out_buf;
-    // k_fft_uneven, contiguous input: 0 = lines land as rows of L and the
-    // first stage maps threads along a line; > 0 = rows of land_row elements
-    // and the first stage maps threads across lines (tiles of 2 to 8 lines).
-    int land_row;
     // Batched uneven lengths in one launch (k_fft_uneven_one): dependency
     // slot s + 1 whose finished-tile counter this job's tiles raise (four-step
     // columns), or that it waits for (four-step rows) until the counter
@@ -100,6 +96,16 @@ struct PassDesc {
     // k 2^in_tl + n mod 2^in_tl).
     int in_tl;
     int out_blk;  // four-step columns: 1 = write such blocks
+    // k_fft_uneven: multiply-high reciprocal of L / radix[s] (0 when that is
+    // 1), the exchange buffer stage s reads (row stride, extra values after
+    // every block of ns[s], step between a butterfly's inputs: MrConfig),
+    // where the second buffer and the tile's four-step factors start.
+    unsigned lr_mag[kMrMaxStages];
+    int xrow[kMrMaxStages];
+    int xpad[kMrMaxStages];
+    int xstep[kMrMaxStages];
+    int xbuf;
+    int ptw_at;
 };
 
 // Fill ns[] (product of the earlier radices) and its multiply-high

@@ -361,7 +361,8 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
     int* tiles = tile_scratch_of(sl);
     struct Group {
         bool fwd;
-        int job0, njobs, tile0, land, work;
+        int job0, njobs, tile0;
+        size_t smem;
         long long ntiles;
     };
     Group groups[kBatchGroups];
@@ -370,7 +371,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
     for (int ph = 0; ph < phases; ++ph) {
         for (int dir = 0; dir < 2; ++dir) {
             const bool fwd = dir == 0;
-            Group g{fwd, nj, 0, nt, 16, 16, 0};
+            Group g{fwd, nj, 0, nt, 0, 0};
             for (size_t i = 0; i < sl.reqs.size(); ++i) {
                 const Req& r = sl.reqs[i];
                 if ((r.direction == FB_FFT_FORWARD) != fwd) continue;
@@ -394,8 +395,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
                     d.apply_scale = (j.last && scale) ? 1 : 0;
                     tiles[nt++] = (int)g.ntiles;
                     g.ntiles += j.d.ntiles;
-                    g.land = std::max(g.land, j.land);
-                    g.work = std::max(g.work, j.work);
+                    g.smem = std::max(g.smem, j.smem);
                     ++nj;
                     ++g.njobs;
                 }
@@ -430,9 +430,9 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
         const Group& g = groups[k];
         const int rc = g.njobs <= kUnevenInlineJobs
                            ? host::batch_launch_inline(g.fwd, jobs + g.job0, packed_tiles + g.tile0, g.njobs,
-                                                       g.ntiles, g.land, g.work, sl.stream)
-                           : host::batch_launch(g.fwd, djobs + g.job0, dtiles + g.tile0, g.njobs, g.ntiles, g.land,
-                                                g.work, sl.stream);
+                                                       g.ntiles, g.smem, sl.stream)
+                           : host::batch_launch(g.fwd, djobs + g.job0, dtiles + g.tile0, g.njobs, g.ntiles, g.smem,
+                                                sl.stream);
         if (rc != FB_FFT_OK) return rc;
     }
     for (size_t i = 0; i < sl.reqs.size(); ++i) {

@@ -26,7 +26,7 @@ cudaError_t uneven_launch_inline(bool forward, const UnevenInlineArgs& a, long l
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kUnevenThreads);
+    cfg.blockDim = dim3(kUnevenBlock);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.numAttrs = 0;
@@ -38,7 +38,7 @@ cudaError_t uneven_occupancy_inline(bool forward, size_t smem, int* blocks_per_s
     const UnevenInlineFn fn = uneven_inline_fn(forward);
     cudaError_t e = kernel_smem_optin((const void*)fn, 0);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)fn, kUnevenThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)fn, kUnevenBlock, smem);
 }
 
 cudaError_t uneven_launch(bool forward, const UnevenArgs& a, long long grid, size_t smem, cudaStream_t stream)
@@ -49,7 +49,7 @@ cudaError_t uneven_launch(bool forward, const UnevenArgs& a, long long grid, siz
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kUnevenThreads);
+    cfg.blockDim = dim3(kUnevenBlock);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.numAttrs = 0;
@@ -61,7 +61,7 @@ cudaError_t uneven_occupancy(bool forward, size_t smem, int* blocks_per_sm)
     const UnevenFn fn = uneven_fn(forward);
     cudaError_t e = kernel_smem_optin((const void*)fn, 0);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)fn, kUnevenThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)fn, kUnevenBlock, smem);
 }
 
 cudaError_t uneven_launch_one(bool forward, const UnevenArgs& a, long long grid, size_t smem, cudaStream_t stream)
@@ -72,7 +72,7 @@ cudaError_t uneven_launch_one(bool forward, const UnevenArgs& a, long long grid,
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kUnevenThreads);
+    cfg.blockDim = dim3(kUnevenBlock);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.numAttrs = 0;
@@ -84,7 +84,7 @@ cudaError_t uneven_occupancy_one(bool forward, size_t smem, int* blocks_per_sm)
     const UnevenFn fn = uneven_one_fn(forward);
     cudaError_t e = kernel_smem_optin((const void*)fn, 0);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)fn, kUnevenThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, (const void*)fn, kUnevenBlock, smem);
 }
 
 }  // namespace fbfft

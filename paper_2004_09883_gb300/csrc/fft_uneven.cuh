@@ -9,26 +9,39 @@
 // offset tables, strides, radix schedule and twiddle tables) sit in a device
 // table; a device prefix table gives each job's first global tile.
 // k_fft_uneven's persistent CTAs walk the global tiles blockIdx.x,
-// +gridDim.x, ... (k_fft_uneven_one's claim them from a counter): the job of a
-// tile is found by walking the prefix table forward (tiles only grow).
-// Two landing buffers, each with its tile's descriptor in shared memory:
-// while tile i is transformed, every thread's cp.async copies bring tile i+1
-// (16-byte copies where the layout allows, else 8-byte).  The stages alternate
-// between the work buffer and the tile's own landing buffer, so every stage
-// needs one barrier; the last stage stores to global memory directly.  Stage
-// radices come from the descriptor (8, 4, 2, 5, 3: at most 10 values of one
-// thread in flight), which keeps the kernel at 64 registers and three
-// buffers, four CTAs per SM.
+// +gridDim.x, ... (k_fft_uneven_one's claim them from a counter).
+//
+// A tile runs as in fft_mr.cuh, with the job's shape read from its descriptor:
+// stages of composite radices up to 16 (two for most lengths up to 256, three
+// above), loads straight from global memory into registers, exchanges through
+// one or two shared-memory buffers, stores straight back.  A control warp beside
+// the eight compute warps walks the job table one tile ahead.
+//
+// What bounds it: latency (issue slots 36 % busy, long scoreboard and barrier
+// stalls; 72 registers leave three CTAs per SM).  On 4096 lengths in [64, 65536]
+// the large radices halved the instructions (417 -> 206 M warp instructions, 180
+// -> 89 per value and pass) and took 565 -> 530 us; with the table walk, claims and
+// counter traffic moved to the control warp 418 us.  256 waiting requests of a
+// server, 2190 -> 1650 us: there the strided tiles of 1000- to 2048-point lines
+// (rows of 2 to 4 values) take most of the time.  Measured without gain: 128
+// compute threads and 2048 values per tile (420 us; the server's long lines then
+// have rows of 1 or 2: 2110), tiles claimed in pairs (434), twiddles read ahead of
+// each stage's barrier (417).
 #pragma once
 
+#include <algorithm>
+
 #include "fft_device.cuh"
+#include "fft_mr.cuh"
 
 namespace fbfft {
 
 constexpr int kUnevenThreads = 256;
-constexpr int kUnevenElems = 8;                                 // values per thread and stage
-constexpr int kUnevenCap = kUnevenThreads * kUnevenElems;       // values per tile (2048)
-constexpr int kUnevenMaxLen = kUnevenCap;                       // longest line of a job
+constexpr int kUnevenCtas = 3;        // per SM: 72 registers, 70 KB of exchange buffers
+constexpr int kUnevenCap = 4096;      // values per tile
+constexpr int kUnevenMaxLen = 2048;   // longest line of a job
+constexpr int kUnevenMaxRadix = 16;
+constexpr int kUnevenMaxLines = 128;  // contiguous lines per tile
 
 // Kernel argument: the job table and the tile prefix table (device memory,
 // written once when the plan is built, or per launch by the request server)
@@ -41,14 +54,14 @@ struct UnevenArgs {
     float2* out;            // buffer 1: the caller's output
     float2* scratch;        // buffer 2: the plan's four-step intermediate
     int njobs;
-    int land_max;           // elements of one landing buffer (multiple of 16; holds a padded work tile too)
-    int work_max;           // elements of the work buffer (multiple of 16)
     int scale_on;           // 1: jobs marked apply_scale multiply by their `scale`
     // One-launch form (k_fft_uneven_one) only: device counters, nsync of
     // them, zero between execs -- [0] tiles claimed, [1] CTAs finished,
-    // [1 + s] finished tiles of dependency slot s (PassDesc::dep_post / dep).
+    // [1 + s] finished tiles of dependency slot s >= 1 (PassDesc::dep_post /
+    // dep), [nsync - 1] finished column tiles of the batch.
     unsigned long long* sync;
     int nsync;
+    int columns;            // column tiles of the batch
     int dep_extra;          // test hook: added to every dependency target (the waits then run out)
 };
 
@@ -73,16 +86,10 @@ __device__ __forceinline__ UTileIdx utile_index(const PassDesc& d, int tile)
     UTileIdx ti;
     const int tpo = (int)d.tiles_per_o;
     ti.o = (int)((unsigned)tile / (unsigned)tpo);
-    ti.c0 = (tile - ti.o * tpo) << d.logT;
+    ti.c0 = (tile - ti.o * tpo) * d.T;
     const int rem = (int)d.C - ti.c0;
-    const int T = 1 << d.logT;
-    ti.Tv = rem < T ? rem : T;
+    ti.Tv = rem < d.T ? rem : d.T;
     return ti;
-}
-
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gsrc) : "memory");
 }
 
 // A job's input / output base in this exec's buffers; kind 3: the field is
@@ -113,42 +120,23 @@ __device__ __forceinline__ float2* uline_out(const UnevenArgs& a, const PassDesc
     return out + (long long)o * d.out_so + (long long)c * d.out_sc;
 }
 
-// Copy tile ti of job d into `land` with cp.async (the caller commits and
-// waits).  Contiguous lines land as [t][n]: 2^lgt threads per line (T <= 256
-// lines, both powers of two), consecutive threads on consecutive values, so a
-// thread finds its line once per tile.  Strided tiles land as [n][t]:
-// consecutive threads on consecutive lines.  Pairs of values move as one
-// 16-byte copy when every address of the tile is 16-byte aligned.
-__device__ __forceinline__ void utile_load(const UnevenArgs& a, const PassDesc& d, const UTileIdx& ti, float2* land)
+// A value of the batch: read once per pass, so its line leaves L1 first.
+__device__ __forceinline__ float2 uload(const float2* p)
 {
-    constexpr int LGTH = 8;  // log2(kUnevenThreads)
-    const int L = d.L, logT = d.logT, tid = threadIdx.x;
-    if (!d.in_tfast) {
-        const int lgt = LGTH - logT, t = tid >> lgt, step = 1 << lgt;
-        if (t >= ti.Tv) return;
-        const float2* src = uline_in(a, d, ti.o, ti.c0 + t);
-        const int lrow = d.land_row ? d.land_row : L;
-        float2* dst = land + t * lrow;
-        if ((L & 1) == 0 && (lrow & 1) == 0 && ((uintptr_t)src & 15) == 0) {
-            for (int n = 2 * (tid & (step - 1)); n < L; n += 2 * step) cp_async16(dst + n, src + n);
-        } else {
-            for (int n = tid & (step - 1); n < L; n += step) cp_async8(dst + n, src + n);
-        }
-    } else {
-        const float2* base = uline_in(a, d, ti.o, ti.c0);
-        const long long sn = d.in_sn;
-        const int T = 1 << logT;
-        if (logT >= 1 && (ti.Tv & 1) == 0 && (sn & 1) == 0 && ((uintptr_t)base & 15) == 0) {
-            const int lg = logT - 1, t = 2 * (tid & ((1 << lg) - 1)), step = kUnevenThreads >> lg;
-            if (t >= ti.Tv) return;
-            for (int n = tid >> lg; n < L; n += step) cp_async16(land + n * T + t, base + n * sn + t);
-        } else {
-            const int t = tid & (T - 1), step = kUnevenThreads >> logT;
-            if (t >= ti.Tv) return;
-            for (int n = tid >> logT; n < L; n += step) cp_async8(land + n * T + t, base + n * sn + t);
-        }
-    }
+    float2 v;
+    asm volatile("ld.global.L1::evict_first.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
 }
+// What the control warp works out about a tile before the compute warps get
+// it: its place (number < 0: no more tiles), its first line's input and
+// output, and where its other contiguous lines start relative to that.
+struct UTile {
+    int number;
+    UTileIdx ti;
+    const float2* in;
+    float2* out;
+    long long line[kUnevenMaxLines];
+};
 
 // exp(-2 pi i m / N) from the job's two split four-step tables (m < N < 2^31).
 __device__ __forceinline__ float2 uptw(const PassDesc& d, unsigned m)
@@ -156,177 +144,227 @@ __device__ __forceinline__ float2 uptw(const PassDesc& d, unsigned m)
     return cmul(__ldg(d.ptw_hi + (m >> d.ptw_log)), __ldg(d.ptw_lo + (m & ((1u << d.ptw_log) - 1))));
 }
 
-// A shared-memory value read with a volatile load (see ustage).
-template <class T>
-__device__ __forceinline__ T uvol(const T& x)
-{
-    return *const_cast<const volatile T*>(&x);
-}
+// Stage twiddles w^r, w = w_{Ns R}^k, of a butterfly at position k (table entry
+// (r-1) Ns + k): small radices read every factor; from 8 on w and every fourth
+// power are read and the others formed by at most three products in a row.
+// Every tile reads its own job's tables, which mostly miss L1: few loads, and
+// those ahead of the barrier the stage starts with.
+template <int R>
+struct UTwiddle {
+    static constexpr int N = R <= 6 ? (R > 1 ? R - 1 : 1) : 1 + (R - 1) / 4;
+    float2 w[N];
+    __device__ __forceinline__ void load(const float2* tw, int Ns)  // tw: the table at k
+    {
+        if constexpr (R > 1) {
+#pragma unroll
+            for (int m = 0; m < N; ++m) w[m] = __ldg(tw + (R <= 6 ? m : (m ? 4 * m - 1 : 0)) * Ns);
+        }
+    }
+    template <bool FWD>
+    __device__ __forceinline__ void apply(float2* v) const
+    {
+        if constexpr (R <= 6) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = twmul<FWD>(v[r], w[r - 1]);
+        } else {
+            const float2 w1 = w[0], w2 = cmul(w1, w1), w3 = cmul(w2, w1);
+            v[1] = twmul<FWD>(v[1], w1);
+            v[2] = twmul<FWD>(v[2], w2);
+            v[3] = twmul<FWD>(v[3], w3);
+#pragma unroll
+            for (int r = 4; r < R; ++r) {
+                const float2 x = w[r / 4];
+                v[r] = twmul<FWD>(v[r], r % 4 == 0 ? x : cmul(x, r % 4 == 1 ? w1 : (r % 4 == 2 ? w2 : w3)));
+            }
+        }
+    }
+};
 
-// One Stockham stage of radix R over the tile (see fft_device.cuh for the
-// formula).  Buffers: stage 0 reads the landing buffer (the input layout) and
-// writes the padded work buffer; from then on the tile's own landing buffer
-// is free and serves as the second work buffer: stage st >= 1 reads the work
-// buffer and writes the landing buffer when st is odd, the other way round
-// when st is even, so no stage waits between its reads and its writes.  The
-// last stage stores straight to global memory (coalesced in both output
-// layouts), with the four-step twiddle and the scale applied.
+// Barrier among the compute warps (named barrier 1).
+__device__ __forceinline__ void usync() { asm volatile("bar.sync 1, %0;" ::"n"(kUnevenThreads) : "memory"); }
+
+// One stage of radix R over the tile, lines and positions as in fft_mr.cuh
+// with the shape read from the descriptor: the first stage loads its
+// butterflies from global memory, stage st >= 1 reads exchange buffer
+// (st - 1) & 1, every stage but the last writes buffer st & 1, the last stores
+// to global memory with the four-step twiddle and the scale applied.
 template <int R, bool FWD, int POS>
-__device__ __forceinline__ void ustage(const UnevenArgs& a, const PassDesc& d, int st, float2* land, float2* work,
-                                       const UTileIdx& ti)
+__device__ __forceinline__ void ustage(const UnevenArgs& a, const PassDesc& d, const UTile& tl, int st, float2* buf)
 {
-    constexpr int LGTH = 8;
-    constexpr int Q = (kUnevenElems + R - 1) / R;
     constexpr bool first = POS == kPosFirst;
     constexpr bool last = POS == kPosLast;
     static_assert(POS == kPosFirst || POS == kPosMid || POS == kPosLast, "stage positions of the uneven kernel");
-    const float2* rd = (st & 1) ? work : land;
-    float2* wr = (st & 1) ? land : work;
-    // Descriptor fields are read afresh in every stage (volatile loads), so
-    // nothing derived from them stays live from one stage to the next.
-    const int L = uvol(d.L), LS = uvol(d.LS), logT = uvol(d.logT);
-    const int LR = L / R;
-    const bool in_tf = first && uvol(d.in_tfast) != 0;
-    const bool out_tf = last && uvol(d.out_tfast) != 0;
-    // contiguous input with padded landing rows: the first stage too maps
-    // threads across lines (its radix-R groups would otherwise fill a
-    // half-warp at stride R)
-    const int lrow = first ? uvol(d.land_row) : 0;
-    const bool tfast = in_tf || out_tf || lrow != 0;
-    const int tid = threadIdx.x;
-    const int lgG = LGTH - logT, G = 1 << lgG;
-    const int t = tfast ? (tid & ((1 << logT) - 1)) : (tid >> lgG);
-    const int jb = tfast ? (tid >> logT) : (tid & (G - 1));
-    const bool tok = t < ti.Tv;
-    float2 v[Q][R];
+    const int L = d.L, logT = d.logT, LR = L / R;
+    const bool in_tf = d.in_tfast != 0, out_tf = d.out_tfast != 0;
+    const bool tf = first ? in_tf : out_tf;
+    const int Tv = tl.ti.Tv, nb = tf ? (LR << logT) : Tv * LR;
+    const unsigned lrm = d.lr_mag[st];
+    const int Ns = first ? 1 : d.ns[st];
+    const unsigned nsm = first ? 0u : d.ns_mag[st];
+    const float2* twb = d.tw + (first ? 0 : d.twoff[st]);
+    const float2* rd = (st & 1) ? buf : buf + d.xbuf;
+    float2* wr = (st & 1) ? buf + d.xbuf : buf;
+    const int rrow = first ? 0 : d.xrow[st], rpad = first ? 0 : d.xpad[st], rstep = first ? 0 : d.xstep[st];
+    const int wrow = last ? 0 : d.xrow[st + 1], wblk = last ? 0 : Ns * R + d.xpad[st + 1];
+    const float2* in0 = first ? tl.in : nullptr;
+    float2* out0 = last ? tl.out : nullptr;
+    const long long sn = first ? (in_tf ? d.in_sn : 1) : (last ? (out_tf ? d.out_sk : 1) : 0);
+    const bool ptw = last && d.ptw != 0, scale = last && a.scale_on && d.apply_scale;
+    const float sc = scale ? d.scale : 1.0f;
+    const int c0 = ptw ? tl.ti.c0 : 0;
+    const float2* p4t = ptw ? buf + d.ptw_at : nullptr;
+    int b = threadIdx.x, t = 0, j = 0, q = 0, k = 0;
+    UTwiddle<R> tw;
+    float2 plo = make_float2(0.f, 0.f), phi = plo;
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int j = jb + q * G;
-        if (tok && j < LR) {
-            if constexpr (first) {
-                if (in_tf) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r) v[q][r] = land[((j + r * LR) << logT) + t];
-                } else {
-                    const float2* p = land + t * (lrow ? lrow : L) + j;
-#pragma unroll
-                    for (int r = 0; r < R; ++r) v[q][r] = p[r * LR];
-                }
-            } else {
-                const float2* p = rd + t * LS + j;
-#pragma unroll
-                for (int r = 0; r < R; ++r) v[q][r] = p[r * LR];
-            }
+    for (int m = 0; m < tw.N; ++m) tw.w[m] = make_float2(0.f, 0.f);
+    auto place = [&]() {  // butterfly b: line t, position j = q Ns + k, and its table reads
+        if (tf) {
+            t = b & ((1 << logT) - 1);
+            j = b >> logT;
         } else {
-            // defined on every path: otherwise the register allocator sees the
-            // values live around the tile loop (loaded and used under the same
-            // condition, which it cannot prove) and keeps every radix's set
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[q][r] = make_float2(0.f, 0.f);
+            t = lrm ? (int)__umulhi((unsigned)b, lrm) : b;
+            j = b - t * LR;
         }
-    }
-    const int Ns = first ? 1 : uvol(d.ns[st]);
-    const unsigned nsm = first ? 0u : (unsigned)uvol(d.ns_mag[st]);
-    const float2* twb = d.tw + (first ? 0 : uvol(d.twoff[st]));
-    float2* dst = nullptr;
-    long long sk = 0;
-    bool sc = false;
-    if constexpr (last) {
-        // line c0 + t of the output (contiguous output), or the tile's first
-        // column plus t (strided output)
-        dst = out_tf ? uline_out(a, d, ti.o, ti.c0) + t : uline_out(a, d, ti.o, ti.c0 + (tok ? t : 0));
-        sk = out_tf ? d.out_sk : 1;
-        sc = a.scale_on && d.apply_scale;
-    }
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int j = jb + q * G;
-        if (tok && j < LR) {
-            const int k = first ? 0 : j - (int)__umulhi((unsigned)j, nsm) * Ns;
-            if constexpr (!first) {
-                // the factors are the powers w^r of w = w_{Ns R}^k (table entry
-                // (r-1) Ns + k): radix 8 loads w and w^4 and forms the other five
-                // by complex multiplies (at most three deep), radix 4 and 5 load w
-                // and w^2 -- fewer loads from tables that mostly miss L1
-                const float2* tw = twb + k;
-                if constexpr (R == 8) {
-                    const float2 w1 = __ldg(tw), w4 = __ldg(tw + 3 * Ns);
-                    const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1);
-                    v[q][1] = twmul<FWD>(v[q][1], w1);
-                    v[q][2] = twmul<FWD>(v[q][2], w2);
-                    v[q][3] = twmul<FWD>(v[q][3], w3);
-                    v[q][4] = twmul<FWD>(v[q][4], w4);
-                    v[q][5] = twmul<FWD>(v[q][5], cmul(w4, w1));
-                    v[q][6] = twmul<FWD>(v[q][6], cmul(w4, w2));
-                    v[q][7] = twmul<FWD>(v[q][7], cmul(w4, w3));
-                } else if constexpr (R == 4 || R == 5) {
-                    const float2 w1 = __ldg(tw), w2 = __ldg(tw + Ns);
-                    v[q][1] = twmul<FWD>(v[q][1], w1);
-                    v[q][2] = twmul<FWD>(v[q][2], w2);
-                    v[q][3] = twmul<FWD>(v[q][3], cmul(w2, w1));
-                    if constexpr (R == 5) v[q][4] = twmul<FWD>(v[q][4], cmul(w2, w2));
-                } else {
-#pragma unroll
-                    for (int r = 1; r < R; ++r) v[q][r] = twmul<FWD>(v[q][r], __ldg(tw + (r - 1) * Ns));
-                }
-            }
-            dft<R, FWD>(v[q]);
-            const int base = (j - k) * R + k;
-            if constexpr (!last) {
-                float2* p = wr + t * LS + base;
-#pragma unroll
-                for (int r = 0; r < R; ++r) p[r * Ns] = v[q][r];
-            } else {
-                // last stage: Ns = L / R, so base = j and kk = j + r Ns.  The
-                // four-step twiddle exp(-2 pi i c kk / N) is read from the split
-                // tables for r = 0 and stepped by exp(-2 pi i c Ns / N) for the
-                // rest (at most 7 products in a row): one gather per butterfly
-                const unsigned c = (unsigned)(ti.c0 + t);
-                const bool ptw = d.ptw != 0;
-                float2 w = make_float2(1.f, 0.f), wstep = make_float2(1.f, 0.f);
-                if (ptw && R > 1) wstep = uptw(d, c * (unsigned)Ns);
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int kk = base + r * Ns;
-                    float2 y = v[q][r];
-                    if (ptw) {
-                        w = r == 0 ? uptw(d, c * (unsigned)kk) : cmul(w, wstep);
-                        y = twmul<FWD>(y, w);
-                    }
-                    if (sc) y = d.scale * y;
-                    dst[kk * sk] = y;
-                }
-            }
+        if constexpr (last) {
+            k = j;  // Ns = L / R
+        } else if constexpr (first) {
+            q = j;
+        } else {
+            q = (int)__umulhi((unsigned)j, nsm);
+            k = j - q * Ns;
         }
+        if constexpr (!first) tw.load(twb + k, Ns);
+        if (ptw && t < Tv) {
+            const unsigned m = (unsigned)(c0 + t) * (unsigned)j;  // below N: c0 + t < C
+            phi = __ldg(d.ptw_hi + (m >> d.ptw_log));
+            plo = __ldg(d.ptw_lo + (m & ((1u << d.ptw_log) - 1)));
+        }
+    };
+    if constexpr (!first) usync();
+    if (b < nb) place();
+    while (b < nb) {
+        if (t < Tv) {
+        float2 v[R];
+        if constexpr (first) {
+            const float2* p = in0 + (in_tf ? j * sn + t : tl.line[t] + j);
+            const long long step = LR * sn;
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = uload(p + r * step);
+        } else {
+            const float2* p = rd + t * rrow + j + q * rpad;
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = p[r * rstep];
+            tw.template apply<FWD>(v);
+        }
+        mr_dft<R, FWD>(v);
+        if constexpr (!last) {
+            float2* p = wr + t * wrow + q * wblk + k;
+#pragma unroll
+            for (int r = 0; r < R; ++r) p[r * Ns] = v[r];
+        } else {
+            // the outputs of butterfly j are j + r Ns
+            float2* p = out0 + (out_tf ? j * sn + t : tl.line[t] + j);
+            const long long step = Ns * sn;
+            if (ptw) {
+                // exp(-2 pi i c (j + r Ns) / N): one table product per butterfly
+                // times the tile's own factor exp(-2 pi i c r Ns / N)
+                const float2 w = cmul(phi, plo);
+                const float2* p4 = p4t + t;
+                v[0] = twmul<FWD>(v[0], w);
+#pragma unroll
+                for (int r = 1; r < R; ++r) v[r] = twmul<FWD>(v[r], cmul(w, p4[r << logT]));
+            }
+            if (scale) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] = sc * v[r];
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) p[r * step] = v[r];
+        }
+        }
+        b += kUnevenThreads;
+        if (b < nb) place();
     }
 }
 
-// First or last stage: any radix of the schedule.
+// Stage st, any radix of a schedule.
 template <bool FWD, int POS>
-__device__ __forceinline__ void ustage_any(const UnevenArgs& a, const PassDesc& d, int st, float2* land,
-                                           float2* work, const UTileIdx& ti)
+__device__ __forceinline__ void ustage_any(const UnevenArgs& a, const PassDesc& d, const UTile& tl, int st, float2* buf)
 {
     switch (d.radix[st]) {
-    case 8: ustage<8, FWD, POS>(a, d, st, land, work, ti); break;
-    case 4: ustage<4, FWD, POS>(a, d, st, land, work, ti); break;
-    case 5: ustage<5, FWD, POS>(a, d, st, land, work, ti); break;
-    case 3: ustage<3, FWD, POS>(a, d, st, land, work, ti); break;
-    case 2: ustage<2, FWD, POS>(a, d, st, land, work, ti); break;
-    default:  // radix 1: a copy (length 1, and the stage that ends a one-radix schedule)
-        ustage<1, FWD, POS>(a, d, st, land, work, ti);
+#define FB_USTAGE(R) \
+    case R: ustage<R, FWD, POS>(a, d, tl, st, buf); break;
+        FB_USTAGE(2)
+        FB_USTAGE(3)
+        FB_USTAGE(4)
+        FB_USTAGE(5)
+        FB_USTAGE(6)
+        FB_USTAGE(8)
+        FB_USTAGE(9)
+        FB_USTAGE(10)
+        FB_USTAGE(12)
+        FB_USTAGE(15)
+        FB_USTAGE(16)
+#undef FB_USTAGE
+    default:  // radix 1: a copy (one-radix schedules)
+        ustage<1, FWD, POS>(a, d, tl, st, buf);
         break;
     }
 }
-// Middle stages of radix R, from stage s while the schedule has that radix
-// (schedules list their radices in the order 8, 4, 2, 5, 3).
-template <int R, bool FWD>
-__device__ __forceinline__ void ustage_run(const UnevenArgs& a, const PassDesc& d, int& s, int nst, float2* land,
-                                           float2* work, const UTileIdx& ti)
+// Every stage of tile tl of job d, by the compute warps.
+template <bool FWD>
+__device__ __forceinline__ void utile_run(const UnevenArgs& a, const PassDesc& d, const UTile& tl, float2* buf)
 {
-    while (s < nst - 1 && d.radix[s] == R) {
-        ustage<R, FWD, kPosMid>(a, d, s, land, work, ti);
-        __syncthreads();
-        ++s;
+    ustage_any<FWD, kPosFirst>(a, d, tl, 0, buf);
+    if (d.ptw) {  // four-step columns: the factors of the tile's lines the last stage needs
+        const int R = d.radix[d.nst - 1], step = d.ns[d.nst - 1], T = 1 << d.logT;
+        for (int e = threadIdx.x; e < (R << d.logT); e += kUnevenThreads)
+            if ((e & (T - 1)) < tl.ti.Tv)  // c < C: the product stays below N
+                buf[d.ptw_at + e] = uptw(d, (unsigned)(tl.ti.c0 + (e & (T - 1))) * (unsigned)((e >> d.logT) * step));
+    }
+    const int nst = d.nst;  // each stage from here on starts with a barrier
+    for (int s = 1; s < nst - 1; ++s) ustage_any<FWD, kPosMid>(a, d, tl, s, buf);
+    ustage_any<FWD, kPosLast>(a, d, tl, nst - 1, buf);
+}
+
+// Control warp: ask L2 for the values a tile will read.
+__device__ __forceinline__ void uprefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void utile_prefetch(const PassDesc& d, const UTile& tl, int lane)
+{
+    const int Tv = tl.ti.Tv;
+    if (d.in_tfast) {
+        for (int n = lane; n < d.L; n += 32) {
+            const float2* p = tl.in + (long long)n * d.in_sn;
+            uprefetch(p);
+            if ((((uintptr_t)p ^ (uintptr_t)(p + Tv - 1)) >> 7) != 0) uprefetch(p + Tv - 1);
+        }
+    } else {
+        const int per = (d.L + 15) / 16;  // 128-byte lines of a line of values
+        for (int i = lane; i < Tv * per; i += 32) {
+            const int t = i / per;
+            uprefetch(tl.in + tl.line[t] + (i - t * per) * 16);
+        }
+    }
+}
+// Control warp: fill in the tile of job d.
+__device__ __forceinline__ void utile_find(const UnevenArgs& a, const PassDesc& d, int number, UTile& tl, int lane)
+{
+    const UTileIdx ti = utile_index(d, number);
+    const bool in_c = !d.in_tfast, out_c = !d.out_tfast;
+    if (lane == 0) {
+        tl.number = number;
+        tl.ti = ti;
+        tl.in = uline_in(a, d, ti.o, ti.c0);
+        tl.out = uline_out(a, d, ti.o, ti.c0);
+    }
+    if (in_c || out_c) {
+        // contiguous lines: a side's offset table, or its line stride (the same
+        // on both sides where both are contiguous)
+        const long long* off = in_c ? d.off_in : d.off_out;
+        const long long sc = in_c ? d.in_sc : d.out_sc;
+        for (int t = lane; t < ti.Tv; t += 32)
+            tl.line[t] = off ? off[ti.c0 + t] - off[ti.c0] : (long long)t * sc;
     }
 }
 
@@ -341,90 +379,52 @@ __device__ __forceinline__ int utab(const int* p)
         return __ldg(p);
 }
 
-template <bool FWD, bool INL>
-__device__ __forceinline__ void uneven_body(const UnevenArgs& a, const PassDesc* jobs, const int* tile_start)
-{
-    extern __shared__ __align__(128) unsigned char smem_dyn[];
-    unsigned char* smem_raw = smem_dyn + ((128u - (smem_u32(smem_dyn) & 127u)) & 127u);
-    float2* land0 = reinterpret_cast<float2*>(smem_raw);
-    float2* work = land0 + 2 * a.land_max;
-    __shared__ PassDesc sd[2];  // sd[b]: descriptor of the tile in landing buffer b
-    constexpr int TH = kUnevenThreads;
-    const int total = utab<INL>(tile_start + a.njobs);
-    const int step = gridDim.x;
-    auto copy_desc = [&](int job, int b) {
-        const int* src = reinterpret_cast<const int*>(jobs + job);
-        int* dst = reinterpret_cast<int*>(&sd[b]);
-        for (int w = threadIdx.x; w < (int)(sizeof(PassDesc) / 4); w += TH) dst[w] = utab<INL>(src + w);
-    };
-    pdl_start();
-    int g = blockIdx.x;
-    if (g >= total) return;
-    int j = 0;
-    while (g >= utab<INL>(tile_start + j + 1)) ++j;
-    int jstart = utab<INL>(tile_start + j);
-    copy_desc(j, 0);
-    __syncthreads();
-    utile_load(a, sd[0], utile_index(sd[0], g - jstart), land0);
-    cp_async_commit();
-    for (int i = 0; g < total; g += step, ++i) {
-        const int b = i & 1;
-        const int gl = g - jstart;  // this tile within its job
-        const int gn = g + step;
-        if (gn < total) {  // the next tile's job and descriptor, then its copies
-            while (gn >= utab<INL>(tile_start + j + 1)) ++j;
-            jstart = utab<INL>(tile_start + j);
-            copy_desc(j, b ^ 1);
-            __syncthreads();
-            utile_load(a, sd[b ^ 1], utile_index(sd[b ^ 1], gn - jstart), land0 + (b ^ 1) * a.land_max);
-            cp_async_commit();
-            cp_async_wait<1>();  // this tile's copies have landed (the next tile's may still fly)
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        const PassDesc& d = sd[b];
-        float2* land = land0 + b * a.land_max;
-        const UTileIdx ti = utile_index(d, gl);
-        const int nst = d.nst;  // >= 2: the planner ends a one-radix schedule with a radix-1 copy
-        ustage_any<FWD, kPosFirst>(a, d, 0, land, work, ti);
-        __syncthreads();
-        int s = 1;
-        ustage_run<8, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<4, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<2, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<5, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<3, FWD>(a, d, s, nst, land, work, ti);
-        ustage_any<FWD, kPosLast>(a, d, nst - 1, land, work, ti);
-        __syncthreads();  // buffer b and sd[b] are free for the tile after next
-    }
-}
-
-template <bool FWD>
-__global__ void __launch_bounds__(kUnevenThreads, 4) k_fft_uneven(const __grid_constant__ UnevenArgs a)
-{
-    uneven_body<FWD, false>(a, a.jobs, a.tile_start);
-}
-
 // ---------------------------------------------------------------------------
-// Every pass of a batched uneven exec in ONE launch.  The job table holds the
-// single passes and four-step columns, then the four-step rows; a row reads
-// what the columns of its chunk wrote, so it may start only once they are
-// done.  Tiles are claimed in table order from a device counter (one atomic
-// per tile, issued a tile ahead), not assigned round robin: a claimed tile
-// always belongs to a running CTA, so a row tile waits only for column tiles
-// already held by running CTAs, and a column tile never waits (a CTA claims
-// in increasing order, so whatever it holds before a column tile is a column
-// tile too).  No CTA can therefore wait on one that is not resident,
-// whatever else shares the GPU.  A column tile, once stored, raises its
-// chunk's counter (every thread fences its own stores, a barrier, then one
-// release add, at the barrier after the CTA's next first stage); a row tile's
-// inputs load once an acquire read sees the counter at the chunk's
-// column-tile count.  Where the next tile's inputs are not ready when it is
-// claimed, its copies wait until the current tile is done (bounded: past the
-// limit the error word is set and the tile runs anyway).  The last CTA to
-// finish zeroes the counters for the next exec.
+// The CTA: kUnevenThreads compute threads and one control warp.  The control
+// warp walks the tiles one ahead of the compute warps -- it finds the next
+// tile's job, copies its descriptor to shared memory, sees to its
+// dependencies and asks L2 for its values -- so none of those latencies (about
+// ten dependent global accesses a tile) is on the compute warps' path.
+// Hand-over by named barriers: ready[b] (control arrives, compute waits) says
+// slot b holds a tile whose inputs are there, done[b] (compute arrives, control
+// waits) that slot b's tile is finished.  ready[b] also separates the compute
+// warps' use of the exchange buffers from one tile to the next.
+//
+// Tiles are assigned round robin (ONE = false), or (ONE) claimed in table order
+// from a device counter, every pass of a batched uneven exec in ONE launch.  The
+// job table then holds the single passes and four-step columns, then the
+// four-step rows; a row reads what the columns of its chunk wrote, so it may
+// start only once they are done.  A claimed tile always belongs to a running
+// CTA, so a row tile waits only for column tiles already held by running CTAs,
+// and a column tile never waits (a CTA claims in increasing order, so whatever
+// it holds before a column tile is a column tile too; a tile's count is
+// published before the control warp waits for the next tile's inputs).  No CTA
+// can therefore wait on one that is not resident, whatever else shares the GPU.
+// A finished column tile raises its chunk's counter: its stores, done[b], then
+// a fence and a release add by one control lane (the fence is cumulative over
+// what the barrier ordered before it).  A row tile starts once an acquire read
+// sees the counter at the chunk's column-tile count; the last column tile of
+// the batch is counted in `all`, and once a CTA has seen every column done it
+// reads no more counters.  The wait is bounded: past the limit the error word is
+// set and the tile runs anyway.  The last CTA to finish zeroes the counters for
+// the next exec.
 // ---------------------------------------------------------------------------
+template <int ID>
+__device__ __forceinline__ void ubar_sync()
+{
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(kUnevenThreads + 32) : "memory");
+}
+template <int ID>
+__device__ __forceinline__ void ubar_arrive()
+{
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(kUnevenThreads + 32) : "memory");
+}
+// ready[b]: barriers 2, 3; done[b]: 4, 5.
+__device__ __forceinline__ void uready_wait(int b) { b ? ubar_sync<3>() : ubar_sync<2>(); }
+__device__ __forceinline__ void uready_post(int b) { b ? ubar_arrive<3>() : ubar_arrive<2>(); }
+__device__ __forceinline__ void udone_wait(int b) { b ? ubar_sync<5>() : ubar_sync<4>(); }
+__device__ __forceinline__ void udone_post(int b) { b ? ubar_arrive<5>() : ubar_arrive<4>(); }
+
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p)
 {
     unsigned long long v;
@@ -435,28 +435,18 @@ __device__ __forceinline__ void red_release_add_u64(unsigned long long* p, unsig
 {
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-// Thread 0: whether the inputs of job `job` are ready.  `seen` is the last
-// dependency slot this CTA found complete: counters only grow during an
-// exec, and the acquire that found it complete (then a barrier) already
-// orders every later load of the CTA, so that slot needs no further read.
-__device__ __forceinline__ bool udeps_ready(const UnevenArgs& a, const PassDesc* job, int& seen)
+// One lane: whether column tiles number `need` are counted in slot `dep`.
+__device__ __forceinline__ bool udeps_ready(const UnevenArgs& a, int dep, int need)
 {
-    const int dep = __ldg(&job->dep);
-    if (dep == 0 || dep == seen) return true;
-    if (ld_acquire_u64(a.sync + 1 + dep) <
-        (unsigned long long)__ldg(&job->dep_need) + (unsigned long long)a.dep_extra)
-        return false;
-    seen = dep;
-    return true;
+    return ld_acquire_u64(a.sync + 1 + dep) >= (unsigned long long)need + (unsigned long long)a.dep_extra;
 }
-// Thread 0: wait until they are, at most kWaitLimitNs; past it set the error
-// word.  Once the word is set (by any CTA) no wait lasts longer, so a launch
-// whose waits cannot end still ends within about one limit.
-__device__ __forceinline__ void udeps_wait(const UnevenArgs& a, const PassDesc* job, int* err, int& seen)
+// The same, waited for at most kWaitLimitNs; past it set the error word.  Once
+// the word is set (by any CTA) no wait lasts longer, so a launch whose waits
+// cannot end still ends within about one limit.
+__device__ __forceinline__ void udeps_wait(const UnevenArgs& a, int dep, int need, int* err)
 {
-    if (udeps_ready(a, job, seen)) return;
     const unsigned long long t0 = global_ns();
-    while (!udeps_ready(a, job, seen)) {
+    while (!udeps_ready(a, dep, need)) {
         if (*reinterpret_cast<volatile int*>(err) != 0) return;
         if (global_ns() - t0 > kWaitLimitNs) {
             atomicExch(err, 1);
@@ -466,145 +456,126 @@ __device__ __forceinline__ void udeps_wait(const UnevenArgs& a, const PassDesc* 
     }
 }
 
-template <bool FWD>
-__device__ __forceinline__ void uneven_body_one(const UnevenArgs& a)
+template <bool FWD, bool INL, bool ONE>
+__device__ __forceinline__ void uneven_body(const UnevenArgs& a, const PassDesc* jobs, const int* tile_start)
 {
-    extern __shared__ __align__(128) unsigned char smem_dyn[];
-    unsigned char* smem_raw = smem_dyn + ((128u - (smem_u32(smem_dyn) & 127u)) & 127u);
-    float2* land0 = reinterpret_cast<float2*>(smem_raw);
-    float2* work = land0 + 2 * a.land_max;
-    __shared__ PassDesc sd[2];  // sd[b]: descriptor of the tile in landing buffer b
-    __shared__ int s_tk[2];     // claimed tickets, handed from thread 0 to the CTA
-    __shared__ int s_ok;        // 1: the next tile's inputs are ready
-    __shared__ int s_ok0;       // the same for the first tile (s_ok may change before every warp read it)
-    __shared__ int s_last;      // 1: this CTA finished last
-    constexpr int TH = kUnevenThreads;
-    const int tid = threadIdx.x;
-    const PassDesc* jobs = a.jobs;
-    const int* tile_start = a.tile_start;
-    const int total = __ldg(tile_start + a.njobs);
-    auto copy_desc = [&](int job, int b) {
-        const int* src = reinterpret_cast<const int*>(jobs + job);
-        int* dst = reinterpret_cast<int*>(&sd[b]);
-        for (int w = tid; w < (int)(sizeof(PassDesc) / 4); w += TH) dst[w] = __ldg(src + w);
-    };
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    float2* buf = reinterpret_cast<float2*>(smem_dyn);
+    __shared__ PassDesc sd[2];  // the descriptors of two tiles in turn
+    __shared__ UTile s_tile[2];
     pdl_start();
-    if (tid == 0) {
-        s_tk[0] = (int)atomicAdd(a.sync, 1ull);
-        s_tk[1] = (int)atomicAdd(a.sync, 1ull);
-    }
-    __syncthreads();
-    int g = s_tk[0], gn = s_tk[1];
-    int jg = 0;              // job of tile g
-    bool cur_loaded = false; // tile g's copies issued
-    // A column tile is counted one tile late, at the barrier after the next
-    // tile's first stage: a fence orders only the fencing thread's own
-    // stores, so every thread fences its share of the counted tile's stores,
-    // then the barrier, then one release add -- by then those stores have
-    // drained and the fences cost little (fencing right after the stores
-    // stalled every column tile).  Pending counts go out before any
-    // dependency wait and after the last tile.
-    int pend = 0;  // dependency slot + 1 of a finished column tile not yet counted
-    int seen = 0;  // thread 0: the last dependency slot + 1 found complete
-    auto flush = [&]() {
-        if (pend) {
-            __threadfence();
-            __syncthreads();
-            if (tid == 0) red_release_add_u64(a.sync + 1 + pend, 1ull);
-            pend = 0;
+    if (threadIdx.x < kUnevenThreads) {
+        for (int b = 0;; b ^= 1) {
+            uready_wait(b);
+            if (s_tile[b].number < 0) return;
+            utile_run<FWD>(a, sd[b], s_tile[b], buf);
+            udone_post(b);
         }
-    };
-    if (g < total) {
-        while (g >= __ldg(tile_start + jg + 1)) ++jg;
-        copy_desc(jg, 0);
-        if (tid == 0) s_ok0 = udeps_ready(a, jobs + jg, seen) ? 1 : 0;
-        __syncthreads();
-        cur_loaded = s_ok0 != 0;
-        if (cur_loaded) utile_load(a, sd[0], utile_index(sd[0], g - __ldg(tile_start + jg)), land0);
-        cp_async_commit();
     }
-    for (int i = 0; g < total; ++i) {
+    // ---- control warp ----
+    const int lane = threadIdx.x & 31;
+    const int total = utab<INL>(tile_start + a.njobs);
+    int j = 0, g = ONE ? 0 : (int)blockIdx.x;
+    int post = 0;           // dependency slot + 1 the running tile raises
+    int seen = 0;           // the last dependency slot + 1 found complete
+    bool all = false;       // every column tile of the batch is known to be done
+    for (int i = 0;; ++i) {
         const int b = i & 1;
-        float2* land = land0 + b * a.land_max;
-        const int gl = g - __ldg(tile_start + jg);  // this tile within its job
-        if (!cur_loaded) {  // inputs not ready when it was claimed: wait, then copy
-            flush();
-            if (tid == 0) udeps_wait(a, jobs + jg, sd[b].err, seen);
-            __syncthreads();
-            utile_load(a, sd[b], utile_index(sd[b], gl), land);
-            cp_async_commit();
+        if constexpr (ONE) {
+            if (lane == 0) g = (int)atomicAdd(a.sync, 1ull);
+            g = __shfl_sync(0xffffffffu, g, 0);
+        } else if (i > 0) {
+            g += (int)gridDim.x;
         }
-        // the ticket of the tile after next, used one iteration later
-        unsigned long long claim = 0;
-        if (tid == 0) claim = atomicAdd(a.sync, 1ull);
-        bool next_loaded = false;
-        int jn = jg;
-        if (gn < total) {  // the next tile's job and descriptor, then its copies when its inputs are ready
-            while (gn >= __ldg(tile_start + jn + 1)) ++jn;
-            copy_desc(jn, b ^ 1);
-            if (tid == 0) s_ok = udeps_ready(a, jobs + jn, seen) ? 1 : 0;
-            __syncthreads();
-            next_loaded = s_ok != 0;
-            if (next_loaded)
-                utile_load(a, sd[b ^ 1], utile_index(sd[b ^ 1], gn - __ldg(tile_start + jn)),
-                           land0 + (b ^ 1) * a.land_max);
-            cp_async_commit();
-            cp_async_wait<1>();  // this tile's copies have landed (the next tile's may still fly)
-        } else {
-            cp_async_wait<0>();
+        const bool has = g < total;
+        int next_post = 0, dep = 0, need = 0;
+        if (has) {
+            // the job of tile g: 32 entries of the prefix table at a time
+            for (;;) {
+                const int e = j + 1 + lane;
+                const unsigned m = __ballot_sync(0xffffffffu, e <= a.njobs && g >= utab<INL>(tile_start + e));
+                j += __popc(m);
+                if (m != 0xffffffffu) break;
+            }
+            const int* src = reinterpret_cast<const int*>(jobs + j);
+            int* dst = reinterpret_cast<int*>(&sd[b]);
+            for (int w = lane; w < (int)(sizeof(PassDesc) / 4); w += 32) dst[w] = utab<INL>(src + w);
+            __syncwarp();
+            utile_find(a, sd[b], g - utab<INL>(tile_start + j), s_tile[b], lane);
+            next_post = sd[b].dep_post;
+            if (ONE && !all && sd[b].dep != seen) dep = sd[b].dep, need = sd[b].dep_need;
+        } else if (lane == 0) {
+            s_tile[b].number = -1;
         }
-        __syncthreads();
-        const PassDesc& d = sd[b];
-        const UTileIdx ti = utile_index(d, gl);
-        const int nst = d.nst;
-        const int post = d.dep_post;
-        ustage_any<FWD, kPosFirst>(a, d, 0, land, work, ti);
-        if (pend) __threadfence();  // the previous column tile's stores (see flush)
-        __syncthreads();
-        if (tid == 0 && pend) red_release_add_u64(a.sync + 1 + pend, 1ull);
-        pend = 0;
-        int s = 1;
-        ustage_run<8, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<4, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<2, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<5, FWD>(a, d, s, nst, land, work, ti);
-        ustage_run<3, FWD>(a, d, s, nst, land, work, ti);
-        ustage_any<FWD, kPosLast>(a, d, nst - 1, land, work, ti);
-        if (tid == 0) s_tk[i & 1] = (int)claim;
-        __syncthreads();  // buffer b and sd[b] are free
-        pend = post;
-        g = gn;
-        jg = jn;
-        gn = s_tk[i & 1];
-        cur_loaded = next_loaded;
+        bool ready = true;
+        if (ONE && dep != 0) {
+            unsigned ok = 0;
+            if (lane == 0) {
+                // every column tile counted (slot 0's own counter): no more reads after this
+                ok = udeps_ready(a, dep, need) ? 1u : 0u;
+                if (ok && ld_acquire_u64(a.sync + a.nsync - 1) >= (unsigned long long)a.columns + a.dep_extra) ok = 2u;
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            ready = ok != 0;
+            all = ok == 2u;
+            if (ready) seen = dep;
+        }
+        __syncwarp();
+        if (ready) {
+            uready_post(b);
+            if (has) utile_prefetch(sd[b], s_tile[b], lane);
+        }
+        if (i > 0) {
+            udone_wait(b ^ 1);
+            if (ONE && post && lane == 0) {
+                __threadfence();
+                red_release_add_u64(a.sync + 1 + post, 1ull);
+                red_release_add_u64(a.sync + a.nsync - 1, 1ull);
+            }
+        }
+        if (!ready) {
+            if (lane == 0) udeps_wait(a, dep, need, sd[b].err);
+            __syncwarp();
+            uready_post(b);
+        }
+        post = next_post;
+        if (!has) break;
     }
-    flush();
-    // the last CTA out zeroes the counters (every other CTA's atomics are
-    // ordered before its finish count by the fences)
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(a.sync + 1, 1ull) == (unsigned long long)gridDim.x - 1 ? 1 : 0;
-        if (s_last) __threadfence();
+    if constexpr (ONE) {
+        // the last CTA out zeroes the counters (every other CTA's atomics are
+        // ordered before its finish count by the fences)
+        unsigned last = 0;
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(a.sync + 1, 1ull) == (unsigned long long)gridDim.x - 1 ? 1u : 0u;
+            if (last) __threadfence();
+        }
+        if (__shfl_sync(0xffffffffu, last, 0))
+            for (int k = lane; k < a.nsync; k += 32) a.sync[k] = 0ull;
     }
-    __syncthreads();
-    if (s_last)
-        for (int k = tid; k < a.nsync; k += TH) a.sync[k] = 0ull;
+}
+
+constexpr int kUnevenBlock = kUnevenThreads + 32;
+
+template <bool FWD>
+__global__ void __launch_bounds__(kUnevenBlock, kUnevenCtas) k_fft_uneven(const __grid_constant__ UnevenArgs a)
+{
+    uneven_body<FWD, false, false>(a, a.jobs, a.tile_start);
 }
 
 template <bool FWD>
-__global__ void __launch_bounds__(kUnevenThreads, 4) k_fft_uneven_one(const __grid_constant__ UnevenArgs a)
+__global__ void __launch_bounds__(kUnevenBlock, kUnevenCtas) k_fft_uneven_one(const __grid_constant__ UnevenArgs a)
 {
-    uneven_body_one<FWD>(a);
+    uneven_body<FWD, false, true>(a, a.jobs, a.tile_start);
 }
 
 // The same pass with its job and tile-prefix tables inside the kernel
 // parameter (at most kUnevenInlineJobs jobs): a small batch then needs no
 // copy of its tables to the device before it can start.
 template <bool FWD>
-__global__ void __launch_bounds__(kUnevenThreads, 4) k_fft_uneven_inline(const __grid_constant__ UnevenInlineArgs p)
+__global__ void __launch_bounds__(kUnevenBlock, kUnevenCtas) k_fft_uneven_inline(const __grid_constant__ UnevenInlineArgs p)
 {
-    uneven_body<FWD, true>(p.a, p.jobs, p.tile_start);
+    uneven_body<FWD, true, false>(p.a, p.jobs, p.tile_start);
 }
 
 #endif  // __CUDACC__
@@ -617,12 +588,59 @@ cudaError_t uneven_launch_inline(bool forward, const UnevenInlineArgs& a, long l
 cudaError_t uneven_occupancy_inline(bool forward, size_t smem, int* blocks_per_sm);
 cudaError_t uneven_launch_one(bool forward, const UnevenArgs& a, long long grid, size_t smem, cudaStream_t stream);
 cudaError_t uneven_occupancy_one(bool forward, size_t smem, int* blocks_per_sm);
-inline size_t uneven_smem_bytes(int land_max, int work_max)
+
+// Schedules of every line length of the engine, worked out once per process.
+inline const MrSchedule& uneven_schedule(int L, bool contiguous)
 {
-    return 128 + (size_t)(2LL * land_max + work_max) * sizeof(float2);
+    struct Table {
+        MrSchedule s[2][kUnevenMaxLen + 1] = {};
+        Table()
+        {
+            for (int n = 2; n <= kUnevenMaxLen; ++n) {
+                int m = n;
+                for (int p : {2, 3, 5})
+                    while (m % p == 0) m /= p;
+                if (m == 1)
+                    for (int k = 0; k < 2; ++k) s[k][n] = mr_schedule(n, k != 0, kUnevenMaxRadix);
+            }
+        }
+    };
+    static const Table table;
+    return table.s[contiguous ? 1 : 0][L];
 }
 
-// Row stride (elements) of a tile's work rows (rows are not padded inside):
+// Shape of a job of L-point lines (C per outer index) on the one-kernel
+// batched-uneven engine: the composite-radix schedule of radices up to 16, and
+// as many lines per tile as fit 4096 values -- any number of contiguous lines
+// (at most 128), a power of two where a side is strided (rows of
+// T consecutive values: 16, or 32 for short lines, whatever fits).
+inline MrConfig uneven_shape(long long L, long long C, int io)
+{
+    MrConfig c{};
+    c.L = (int)L, c.io = io;
+    const MrSchedule& s = uneven_schedule((int)L, io == 0);
+    c.n = L == 1 ? 2 : s.n;  // one point: two copies
+    for (int i = 0, ns = 1; i < c.n; ++i) {
+        c.radix[i] = L == 1 ? 1 : s.radix[i];
+        c.ns[i] = ns;
+        ns *= c.radix[i];
+    }
+    auto floor2 = [](long long x) {
+        long long p = 1;
+        while (p * 2 <= x) p *= 2;
+        return p;
+    };
+    long long T = std::max(1LL, kUnevenCap / L);
+    if (io == 0)  // contiguous on both sides
+        T = std::min<long long>(std::min<long long>(T, kUnevenMaxLines), C);
+    else
+        T = std::min(std::min(floor2(T), L <= 64 ? 32LL : 16LL), C <= 1 ? 1LL : 2 * floor2(C - 1));
+    c.T = (int)std::max(1LL, T);
+    return c;
+}
+
+// Row placement rules for tiles of a power of two of lines.  Row stride
+// (elements) of a tile's work rows (rows are not padded inside):
 // at least L, and chosen so that the 16 threads of a half-warp never meet on
 // one bank of 8-byte words across rows.  A stage that maps consecutive
 // threads to consecutive lines (the strided sides of four-step jobs) puts
@@ -650,6 +668,8 @@ inline int uneven_line_stride(long long L, long long T, bool cfast)
 // (stride mod 2H == H, even, so the 16-byte copies stay aligned) and their
 // first stage maps threads across lines: its radix-R groups would otherwise
 // fill a half-warp at stride R (8-way for radix 8).
+// (The kernel's tiles load straight into registers now; the rule stands for
+// tiles that land in rows.)
 inline int uneven_land_row(long long L, long long T, bool in_tfast)
 {
     if (in_tfast || T < 2 || T > 8) return 0;

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "fft_mr.cuh"
+#include "fft_uneven.cuh"
 
 using namespace fbfft;
 using cd = std::complex<double>;
@@ -176,5 +177,27 @@ int main()
         }
     }
     std::printf("row_blocks %lld %lld 0\n", cases, bad);
+    // the jobs of the batched-uneven kernel: run-time shapes, tiles of few lines
+    cases = bad = 0;
+    err = 0;
+    for (int L = 1; L <= kUnevenMaxLen; ++L) {
+        int n = L;
+        for (int p : {2, 3, 5})
+            while (n % p == 0) n /= p;
+        if (n != 1) continue;
+        for (int io = 0; io < 4; ++io)
+            for (long long C : {1LL, 5LL, 100000LL}) {
+                MrConfig c = uneven_shape(L, C, io);
+                bad += c.n < 2 || c.n > kMrMaxStages;
+                mr_place(c);
+                bad += io != 0 && (c.T & (c.T - 1)) != 0;
+                bad += c.T < 1 || c.T > kUnevenThreads || (long long)c.T * L > kUnevenCap;
+                bad += (c.buf[0] + c.buf[1] + c.ptw) * 8 + 2 * (sizeof(PassDesc) + sizeof(UTile)) + 1024 > 233472 / kUnevenCtas;
+                bad += run_tile<true>(c, c.T, &err);
+                bad += run_tile<false>(c, (c.T + 1) / 2, &err);
+                ++cases;
+            }
+    }
+    std::printf("uneven_jobs %lld %lld %.3e\n", cases, bad, err);
     return 0;
 }
