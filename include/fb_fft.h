@@ -407,11 +407,13 @@ int fb_fft_server_create(fb_fft_server_t* srv, int slots, long long hbm_cap_byte
  * the memory budget holds them, at most max_requests and 1024 jobs) run
  * together: their job descriptors, with each request's own addresses, go to
  * the device in one copy and run as one launch per phase and direction (at
- * most six launches for the whole batch).  The batch grows with the queue:
+ * most six launches for the whole batch); 1-D lengths with a four-step factor
+ * above 512 points, each large enough to fill the GPU, run their plan's two
+ * passes beside them, in any batch and alone.  The batch grows with the queue:
  * a request that finds a slot free starts at once, alone.  Results do not
  * depend on what else is in the batch (same bits alone and in any batch);
- * they can differ in the last bits from the per-request path, which uses the
- * plan's own kernels.
+ * those of the job table can differ in the last bits from the per-request
+ * path, which uses the plan's own kernels.
  *   max_requests  <= 1: no batching, every request runs alone through its
  *                 shape's plan (the per-call kernels).  Applies to requests
  *                 submitted after the call.

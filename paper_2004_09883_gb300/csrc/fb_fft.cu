@@ -1596,6 +1596,7 @@ int recipe_create(BatchRecipe** out, int rank, const long long* dims, long long 
         r->jobs.push_back(j);
         r->phases = std::max(r->phases, q.group + 1);
         r->tiles += q.d.ntiles;
+        if (q.io != kIoNN) r->rows = std::min(r->rows, q.d.T);
     }
     *out = r;
     return FB_FFT_OK;

@@ -44,6 +44,7 @@ struct BatchRecipe {
     long long scratch_bytes = 0;  // four-step intermediate of one request
     long long table_bytes = 0;    // device bytes the recipe holds
     long long tiles = 0;          // tiles of all its jobs
+    int rows = 32;                // shortest row of values a strided tile of its jobs moves
     float scale = 1.f;            // 1 / (elements of one transform)
     float2* tw = nullptr;
 };

@@ -21,7 +21,8 @@
 // of such requests that fits the budget (up to max_batch), writes their jobs
 // with the requests' own addresses into the slot's pinned job table, copies
 // it to the device with one copy and runs it as one launch per phase and
-// direction (at most six).  Host work per request is then filling two or
+// direction (at most six); long 1-D lengths run their plan's passes beside
+// them (kBatchRows).  Host work per request is then filling two or
 // three descriptors instead of encoding tensor maps and launching kernels;
 // the batch grows by itself with the queue, so an idle server still starts
 // each request at once.
@@ -118,11 +119,23 @@ struct ShapeKey {
 struct PlanEntry {
     fb_fft_plan_t plan = nullptr;
     host::BatchRecipe* recipe = nullptr;  // null: this shape runs per request
+    // In a batch this shape's requests run their plan's own passes instead of
+    // its recipe's jobs (long 1-D lengths, see kBatchRows)
+    bool by_plan = false;
     unsigned flags = 0;
     long long scratch = 0, io = 0, table = 0;
     long long last_use = 0;
     int users = 0;  // queued + running requests holding it
 };
+
+// Four-step jobs whose strided tiles move rows of fewer values than this (64
+// bytes; factors above 512 points) spend most of the one-kernel engine's load and
+// store path on pieces of a sector or less; such a request fills the GPU by
+// itself, and its plan's two launches, whose tiles are wider or moved by the copy
+// engine, run it faster.  256 waiting requests, 81 % of whose values are in such
+// lengths: 1637 us with none of them by plan, 1264 with rows of fewer than 4
+// values (factors above 1024), 1235 with fewer than 8.
+constexpr int kBatchRows = 8;
 
 // Jobs one slot's table holds (a batch of up to 1024 jobs: 341 four-step or
 // 3-D requests, more of the others).
@@ -227,6 +240,7 @@ int get_plan(fb_fft_server_s* s, int rank, const long long* dims, long long batc
             e.recipe = nullptr;
         }
         if (e.recipe) e.table += e.recipe->table_bytes;
+        e.by_plan = e.recipe && rank == 1 && e.recipe->rows < kBatchRows;
         // the twiddle tables are written on the build stream; requests run on
         // the slots' streams, so the tables must be complete before the first
         const cudaError_t se = cudaStreamSynchronize(s->build);
@@ -248,7 +262,7 @@ long long up_align(long long n) { return (n + kArenaAlign - 1) / kArenaAlign * k
 
 long long scratch_of(const PlanEntry* pe, bool batched)
 {
-    return batched ? pe->recipe->scratch_bytes : pe->scratch;
+    return batched && !pe->by_plan ? pe->recipe->scratch_bytes : pe->scratch;
 }
 
 long long request_need(const PlanEntry* pe, bool host_io, bool batched)
@@ -352,8 +366,9 @@ int* tile_scratch_of(Slot& sl)
 
 // Put the batch on slot sl: its job table (every request's jobs with their
 // addresses, grouped by phase and direction, each group with its tile
-// prefixes) goes to the device in one copy, then one launch per group, all on
-// the slot's stream, between the slot's two events.
+// prefixes) goes to the device in one copy, then one launch per group, behind
+// the plan passes of the requests that run by plan, all on the slot's stream,
+// between the slot's two events.
 int start_batch(fb_fft_server_s* s, Slot& sl)
 {
     // jobs first; the tile prefixes go right behind the last job (one copy)
@@ -376,6 +391,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
                 const Req& r = sl.reqs[i];
                 if ((r.direction == FB_FFT_FORWARD) != fwd) continue;
                 char* block = sl.offs[i] >= 0 ? s->arena.base + sl.offs[i] : nullptr;
+                if (r.pe->by_plan) continue;
                 const long long scr = up_align(r.pe->recipe->scratch_bytes);
                 // host arrays: the transform runs in place in the staging buffer
                 const float2* in = r.host_io ? reinterpret_cast<const float2*>(block + scr)
@@ -412,8 +428,17 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
     for (size_t i = 0; i < sl.reqs.size(); ++i) {
         const Req& r = sl.reqs[i];
         if (!r.host_io) continue;
-        char* stage = s->arena.base + sl.offs[i] + up_align(r.pe->recipe->scratch_bytes);
+        char* stage = s->arena.base + sl.offs[i] + up_align(scratch_of(r.pe, true));
         SV_CK(cudaMemcpyAsync(stage, r.in, (size_t)r.pe->io, cudaMemcpyHostToDevice, sl.stream));
+    }
+    for (size_t i = 0; i < sl.reqs.size(); ++i) {
+        const Req& r = sl.reqs[i];
+        if (!r.pe->by_plan) continue;
+        char* block = sl.offs[i] >= 0 ? s->arena.base + sl.offs[i] : nullptr;
+        char* stage = block + up_align(scratch_of(r.pe, true));
+        const int rc = host::plan_exec_on(r.pe->plan, r.host_io ? stage : r.in, r.host_io ? stage : r.out, r.direction,
+                                          sl.stream, block, sl.err_dev);
+        if (rc != FB_FFT_OK) return rc;
     }
     int* packed_tiles = reinterpret_cast<int*>(sl.tab_host + (size_t)nj * sizeof(PassDesc));
     std::memmove(packed_tiles, tiles, (size_t)nt * sizeof(int));
@@ -438,7 +463,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
     for (size_t i = 0; i < sl.reqs.size(); ++i) {
         const Req& r = sl.reqs[i];
         if (!r.host_io) continue;
-        const char* stage = s->arena.base + sl.offs[i] + up_align(r.pe->recipe->scratch_bytes);
+        const char* stage = s->arena.base + sl.offs[i] + up_align(scratch_of(r.pe, true));
         SV_CK(cudaMemcpyAsync(r.out, stage, (size_t)r.pe->io, cudaMemcpyDeviceToHost, sl.stream));
     }
     if (!sl.err_mapped)
