@@ -139,6 +139,9 @@ for _name, (_res, _args) in _sig.items():
     _f.argtypes = _args
 
 
+_exec = lib.fb_fft_exec
+
+
 def _text(status: int) -> str:
     return lib.fb_fft_status_string(int(status)).decode()
 
@@ -209,6 +212,24 @@ def twiddles(d: int, count: int) -> np.ndarray:
     return out.view(np.complex64)
 
 
+# torch and its raw current-stream getter, bound by the first device call: a
+# small transform's call is bound by this binding (4096 points x 64, back to
+# back: 8.0 us a call through torch's stream objects and ctypes pointer objects,
+# 5.2 with these; the kernel itself takes 5.2).
+_torch = None
+_raw_stream = None
+
+
+def _bind_torch():
+    """Import torch for the device calls (the host-only functions work without)."""
+    global _torch, _raw_stream
+    import torch
+    get = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    _raw_stream = get or (lambda index: torch.cuda.current_stream(index).cuda_stream)
+    _torch = torch
+    return torch
+
+
 def _stream_handle(stream) -> int:
     if stream is None:
         import torch
@@ -270,19 +291,22 @@ class Plan:
     def exec(self, x, out=None, direction: int = FORWARD):
         """Transform torch complex64 CUDA tensor ``x`` (batch*prod(dims) values)
         into ``out`` (new tensor if None; ``out is x`` runs in place)."""
-        import torch
+        torch = _torch or _bind_torch()
         if x.dtype != torch.complex64 or not x.is_cuda or not x.is_contiguous():
             raise ValueError("x must be a contiguous complex64 CUDA tensor")
-        if x.numel() != self.n * self.batch:
-            raise ValueError(f"x has {x.numel()} values, plan expects {self.n * self.batch}")
+        count = x.numel()
+        if count != self.n * self.batch:
+            raise ValueError(f"x has {count} values, plan expects {self.n * self.batch}")
         if out is None:
             out = torch.empty_like(x)
-        elif out.dtype != torch.complex64 or not out.is_contiguous() or out.numel() != x.numel():
+        elif out.dtype != torch.complex64 or not out.is_contiguous() or out.numel() != count:
             raise ValueError("out must be a contiguous complex64 tensor like x")
-        s = torch.cuda.current_stream(x.device).cuda_stream
+        s = _raw_stream(x.get_device())
         if s != self._stream:
             self.set_stream(s)
-        self.exec_ptr(x.data_ptr(), out.data_ptr(), direction)
+        rc = _exec(self._h, x.data_ptr(), out.data_ptr(), int(direction))
+        if rc:
+            raise FFTError(rc, "fb_fft_exec")
         return out
 
     def exec_host(self, x: np.ndarray, out: np.ndarray | None = None, direction: int = FORWARD):
