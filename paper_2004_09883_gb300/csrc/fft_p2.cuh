@@ -125,7 +125,7 @@ __host__ __device__ constexpr long long p2_smem_bytes(int threads, int lg, int i
     return 256 + 8LL * (p2_land_elems(threads, lg, io) * (async ? p2_nbuf(threads) : 1) +
                         (pow2_nst(lg) > 1 ? (long long)p2_work_stride(threads, lg, io) * p2_tile_lines(threads, lg, io) : 0) +
                         (tc ? 0 : p2_smem_twiddles(lg))) +
-           (tc ? (long long)kTcExtraSmem : 0);
+           (tc ? (long long)kTcExtraSmem + (io == kIoCCP ? 16 * 8LL * p2_tile_lines(threads, lg, io) : 0) : 0);
 }
 
 template <int THREADS, int LG, int IO>
@@ -326,13 +326,36 @@ __device__ __forceinline__ void p2_stage(const PassDesc& d, float2* land, float2
     }
 }
 
+// exp(-2 pi i m / N) from the split four-step tables (m < N < 2^31).
+__device__ __forceinline__ float2 p2_ptw(const PassDesc& d, unsigned m)
+{
+    return cmul(__ldg(d.ptw_hi + (m >> d.ptw_log)), __ldg(d.ptw_lo + (m & ((1u << d.ptw_log) - 1))));
+}
+// Tensor-core four-step columns: the factors exp(-2 pi i c r LR / N) of a tile's
+// lines c = c0 + t, at [r T + t], for the last stage (a barrier away).  With
+// every output's factor gathered from the tables of N, two reads a value, 2^20
+// x 32 took 308 us; with these and the stage twiddles read ahead of their
+// barrier (p2_tc_twiddles) 287, at the same error (8.5e-7).  Stepping from factor
+// to factor as the FP32 stage does: 276 us, but 8.6e-7.  The FP32 columns measured
+// slower with such a table (211.4 against 208.7 us).
+template <int THREADS, int LG, int IO>
+__device__ __forceinline__ void p2_tc_ptw(const PassDesc& d, int Tv, int c0, const TcState& tc)
+{
+    using C = P2<THREADS, LG, IO>;
+    if constexpr (C::PTW) {
+        for (int e = threadIdx.x; e < 16 * C::T; e += THREADS)
+            if ((e & (C::T - 1)) < Tv)  // c < C: the product stays below N
+                tc.ptw[e] = p2_ptw(d, (unsigned)(c0 + (e & (C::T - 1))) * (unsigned)((e >> C::LOGT) * (C::L / 16)));
+    }
+}
+
 // A radix-16 stage on the tensor cores (fft_tc.cuh): same gather, twiddles
 // and scatter as p2_stage, the 16-point DFT as one FP16 hi/lo matrix product
 // per 128 butterflies.  Needs exactly one butterfly per compute thread and at
 // least two stages (the A tiles live in the work buffer).
 template <int THREADS, bool FWD, int LG, int IO, int S>
 __device__ __forceinline__ void p2_stage_tc(const PassDesc& d, float2* land, float2* work, int Tv, int c0,
-                                            const float2* tws, TcState& tc)
+                                            const float2* tws, TcState& tc, const float2 (&twr)[15])
 {
     using C = P2<THREADS, LG, IO>;
     constexpr int L = C::L, T = C::T, G = C::G;
@@ -372,10 +395,9 @@ __device__ __forceinline__ void p2_stage_tc(const PassDesc& d, float2* land, flo
     }
     if constexpr (!first && !kTcATmem) compute_sync<THREADS>();  // A rows overwrite the work buffer just read
     const int k = j & (NS - 1);
-    if constexpr (NS > 1) {  // tensor-core kernels keep the stage twiddles in global memory (L1-cached)
-        const float2* tw = d.tw + d.twoff[S] + k;
+    if constexpr (NS > 1) {
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = twmul<FWD>(v[r], __ldg(tw + (r - 1) * NS));
+        for (int r = 1; r < R; ++r) v[r] = twmul<FWD>(v[r], twr[r - 1]);
     }
     const unsigned abase = smem_u32(work);
     int e;
@@ -394,6 +416,13 @@ __device__ __forceinline__ void p2_stage_tc(const PassDesc& d, float2* land, flo
         else
             tc_issue<THREADS / 128>(tc, abase);
     }
+    // Four-step factors exp(-2 pi i c kk / N) of the outputs kk = j + r LR: one
+    // table product for c j, read while the matrix products run, times the
+    // tile's own factors of c r LR (p2_tc_ptw)
+    float2 w0 = make_float2(1.f, 0.f);
+    if constexpr (last && C::PTW) {
+        if (tok) w0 = p2_ptw(d, (unsigned)(c0 + t) * (unsigned)j);
+    }
     const bool ok = mbar_wait_bounded(tc.bar, tc.uses & 1u);
     tc.uses++;
     if (!ok && (tid & 31) == 0) atomicExch(d.err, 1);
@@ -411,10 +440,7 @@ __device__ __forceinline__ void p2_stage_tc(const PassDesc& d, float2* land, flo
             const int kk = j + r * LR;
             float2 y = v[r];
             if constexpr (C::PTW) {
-                const unsigned m = (unsigned)(c0 + t) * (unsigned)kk;  // < N < 2^31
-                const float2 w = cmul(__ldg(d.ptw_hi + (m >> d.ptw_log)),
-                                      __ldg(d.ptw_lo + (m & ((1u << d.ptw_log) - 1))));
-                y = twmul<FWD>(y, w);
+                y = twmul<FWD>(y, r ? cmul(w0, tc.ptw[r * T + t]) : w0);
             }
             if (d.apply_scale) y = d.scale * y;
             if constexpr (C::OUT_T)
@@ -425,13 +451,31 @@ __device__ __forceinline__ void p2_stage_tc(const PassDesc& d, float2* land, flo
     }
 }
 
+// The twiddles of tensor-core stage S (global memory, L1-cached: a CTA's tables
+// do not fit beside two CTAs' tiles), read ahead of the barrier before it.
+template <int THREADS, int LG, int IO, int S>
+__device__ __forceinline__ void p2_tc_twiddles(const PassDesc& d, float2 (&twr)[15])
+{
+    if constexpr (S < pow2_nst(LG)) {
+        if constexpr (pow2_radix(LG, S) == 16 && pow2_ns(LG, S) > 1) {
+            using C = P2<THREADS, LG, IO>;
+            constexpr bool tfast = S == C::NST - 1 && C::OUT_T;
+            constexpr int NS = pow2_ns(LG, S);
+            const int j = tfast ? (int)(threadIdx.x >> C::LOGT) : (int)(threadIdx.x & (C::G - 1));
+            const float2* tw = d.tw + d.twoff[S] + (j & (NS - 1));
+#pragma unroll
+            for (int r = 1; r < 16; ++r) twr[r - 1] = __ldg(tw + (r - 1) * NS);
+        }
+    }
+}
+
 // Stage S, on the tensor cores when TC and the stage is radix 16.
 template <int THREADS, bool FWD, int LG, int IO, int S, bool TC>
 __device__ __forceinline__ void p2_run_stage(const PassDesc& d, float2* land, float2* work, int Tv, int c0,
-                                             const float2* tws, TcState& tc)
+                                             const float2* tws, TcState& tc, const float2 (&twr)[15])
 {
     if constexpr (TC && pow2_radix(LG, S) == 16) {
-        p2_stage_tc<THREADS, FWD, LG, IO, S>(d, land, work, Tv, c0, tws, tc);
+        p2_stage_tc<THREADS, FWD, LG, IO, S>(d, land, work, Tv, c0, tws, tc, twr);
     } else {
         // tensor-core kernels copy no stage twiddles: their FP32 stage is the first (no twiddles)
         static_assert(!TC || pow2_ns(LG, S) == 1, "FP32 stage with twiddles in a tensor-core kernel");
@@ -441,15 +485,16 @@ __device__ __forceinline__ void p2_run_stage(const PassDesc& d, float2* land, fl
 
 template <int THREADS, bool FWD, int LG, int IO, int S, bool TC>
 __device__ __forceinline__ void p2_stages_from(const PassDesc& d, float2* land, float2* work, int Tv, int c0,
-                                               bool async, const float2* tws, TcState& tc)
+                                               bool async, const float2* tws, TcState& tc, float2 (&twr)[15])
 {
     using C = P2<THREADS, LG, IO>;
     if constexpr (S < C::NST) {
-        p2_run_stage<THREADS, FWD, LG, IO, S, TC>(d, land, work, Tv, c0, tws, tc);
+        p2_run_stage<THREADS, FWD, LG, IO, S, TC>(d, land, work, Tv, c0, tws, tc, twr);
         if constexpr (S == C::NST - 1)
             if (async) fence_proxy_async();  // output tile -> visible to the TMA store
+        if constexpr (TC) p2_tc_twiddles<THREADS, LG, IO, S + 1>(d, twr);
         compute_sync<THREADS>();              // (last stage: the work buffer is free again)
-        p2_stages_from<THREADS, FWD, LG, IO, S + 1, TC>(d, land, work, Tv, c0, async, tws, tc);
+        p2_stages_from<THREADS, FWD, LG, IO, S + 1, TC>(d, land, work, Tv, c0, async, tws, tc, twr);
     }
 }
 
@@ -616,7 +661,7 @@ struct P2Regs {
 // (fft_tc.cuh); the CTA then also holds B^T (4 KB after the work buffer;
 // its stage twiddles stay in global memory)
 // and tc_tmem_cols(THREADS) TMEM columns, allocated by compute warp 0 and
-// freed before it exits.
+// freed before it exits.  Its four-step columns keep 16 factors per line behind B^T.
 template <int THREADS, bool FWD, int LG, int IO, bool TC = false>
 __global__ void __maxnreg__((P2Regs<THREADS, LG>::LAUNCH)) k_fft_p2(const __grid_constant__ LineArgs a)
 {
@@ -682,7 +727,7 @@ __global__ void __maxnreg__((P2Regs<THREADS, LG>::LAUNCH)) k_fft_p2(const __grid
 
     // ---- compute warps ----
     if constexpr (RG::SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(RG::COMPUTE));
-    TcState tc{0u, mma_bar, 0u, 0u, 0u};
+    TcState tc{0u, mma_bar, 0u, 0u, 0u, nullptr};
     if constexpr (TC) {
         unsigned char* bmat = reinterpret_cast<unsigned char*>(
             (reinterpret_cast<uintptr_t>(tws) + 127) & ~static_cast<uintptr_t>(127));
@@ -694,6 +739,7 @@ __global__ void __maxnreg__((P2Regs<THREADS, LG>::LAUNCH)) k_fft_p2(const __grid
         tc_fence_after();
         tc.tmem = *tmem_slot;
         tc.bsm = smem_u32(bmat);
+        tc.ptw = reinterpret_cast<float2*>(bmat + 4096);  // four-step columns: factors of the tile's lines
         tc.a = tc.tmem + 32u * (THREADS / 128);  // A rows after the accumulators
     }
     if constexpr (C::TWS > 0 && !TC) {
@@ -725,13 +771,18 @@ __global__ void __maxnreg__((P2Regs<THREADS, LG>::LAUNCH)) k_fft_p2(const __grid
             p2_plain_load<THREADS, LG, IO>(d, ti, land);
             compute_sync<THREADS>();
         }
-        p2_run_stage<THREADS, FWD, LG, IO, 0, TC>(d, land, work, ti.Tv, c0, tws, tc);
+        float2 twr[15];  // (tensor-core stages only)
+        p2_run_stage<THREADS, FWD, LG, IO, 0, TC>(d, land, work, ti.Tv, c0, tws, tc, twr);
+        if constexpr (TC) {
+            p2_tc_ptw<THREADS, LG, IO>(d, ti.Tv, c0, tc);
+            p2_tc_twiddles<THREADS, LG, IO, 1>(d, twr);
+        }
         if constexpr (C::NST == 1) {
             if (async) fence_proxy_async();
         } else {
             compute_sync<THREADS>();
         }
-        p2_stages_from<THREADS, FWD, LG, IO, 1, TC>(d, land, work, ti.Tv, c0, async, tws, tc);
+        p2_stages_from<THREADS, FWD, LG, IO, 1, TC>(d, land, work, ti.Tv, c0, async, tws, tc, twr);
         if (async) {
             mbar_arrive(&empty[buf]);  // after this thread's proxy fence
         } else {

@@ -170,6 +170,7 @@ struct TcState {
     unsigned bsm;              // shared address of B^T
     unsigned uses;             // completed MMA rounds (mbarrier phase)
     unsigned a;                // TMEM address of the A rows (when kTcATmem)
+    float2* ptw;               // four-step columns: factors of the tile's lines (shared memory)
 };
 
 // The scale exponent of a butterfly: 2^-e brings its largest component into [0.5, 1).
