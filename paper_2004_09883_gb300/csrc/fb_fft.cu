@@ -186,6 +186,7 @@ struct fb_fft_plan_s {
     int rank = 0;
     long long dims[3] = {1, 1, 1};
     long long batch = 0;
+    long long route_batch = 0;  // the batch that chooses the kernels (a chunk plan: the whole batch)
     unsigned flags = 0;
     cudaStream_t stream = nullptr;
     long long N = 1;
@@ -843,10 +844,11 @@ int schedule_plan(fb_fft_plan_s* p, TwiddleBuilder& twb)
             PassPlan q;
             int rc;
             if (S == 1)
-                rc = make_line_pass(q, twb, L, 1, B * Opre, 1, L, 0, 1, L, 0, false, false, false, false, 0, tc);
+                rc = make_line_pass(q, twb, L, 1, B * Opre, 1, L, 0, 1, L, 0, false, false, false, false, 0, tc, false,
+                                    p->route_batch * p->N);
             else
                 rc = make_line_pass(q, twb, L, B * Opre, S, S, 1, L * S, S, 1, L * S, true, true, false, false, 0,
-                                    tc);
+                                    tc, false, p->route_batch * p->N);
             if (rc != FB_FFT_OK) return rc;
             q.src = first ? kBufIn : kBufOut;
             q.dst = kBufOut;
@@ -1326,9 +1328,11 @@ int exec_device(fb_fft_plan_s* p, const float2* in, float2* out, int direction)
 }
 
 // Plan construction shared by fb_fft_plan and the server; ext_scratch plans
-// allocate no scratch (the caller passes one to exec_lines).
+// allocate no scratch (the caller passes one to exec_lines); route_batch is the
+// batch whose kernels the plan takes (0: its own), so that the plan of a part
+// of a batch gives the whole batch's bits.
 int plan_new(fb_fft_plan_s** out, int rank, const long long* dims, long long batch, unsigned flags,
-             cudaStream_t stream, bool ext_scratch)
+             cudaStream_t stream, bool ext_scratch, long long route_batch = 0)
 {
     *out = nullptr;
     long long N = 1;
@@ -1345,6 +1349,7 @@ int plan_new(fb_fft_plan_s** out, int rank, const long long* dims, long long bat
     p->rank = rank;
     for (int d = 0; d < rank; ++d) p->dims[d] = dims[d];
     p->batch = batch;
+    p->route_batch = route_batch > 0 ? route_batch : batch;
     p->flags = flags;
     p->stream = stream;
     p->N = N;
@@ -1412,10 +1417,10 @@ int exec_host_pipelined(fb_fft_plan_s* p, const float2* hin, float2* hout, int d
         free_plan(p->host_tail);
         p->host_chunk = p->host_tail = nullptr;
         p->host_chunk_batch = 0;
-        int rc = plan_new(&p->host_chunk, p->rank, p->dims, cb, p->flags, p->stream, false);
+        int rc = plan_new(&p->host_chunk, p->rank, p->dims, cb, p->flags, p->stream, false, p->batch);
         if (rc != FB_FFT_OK) return rc;
         if (tail != cb) {
-            rc = plan_new(&p->host_tail, p->rank, p->dims, tail, p->flags, p->stream, false);
+            rc = plan_new(&p->host_tail, p->rank, p->dims, tail, p->flags, p->stream, false, p->batch);
             if (rc != FB_FFT_OK) return rc;
         }
         p->host_chunk_batch = cb;

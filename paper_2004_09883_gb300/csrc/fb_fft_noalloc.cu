@@ -165,7 +165,8 @@ int run(const float2* src, float2* dst, long long n, long long batch, bool fwd, 
     StackTwiddles twj;
     if (n <= FB_FFT_MAX_SMEM_LEN) {  // one pass over contiguous lines, no intermediate
         PassPlan p;
-        int rc = make_line_pass(p, twj, n, 1, batch, 1, n, 0, 1, n, 0, false, false, false);
+        int rc = make_line_pass(p, twj, n, 1, batch, 1, n, 0, 1, n, 0, false, false, false, false, 0, false,
+                                (n & (n - 1)) == 0);
         if (rc != FB_FFT_OK) return rc;
         for (int j = 0; j < twj.njobs; ++j)
             if (launch_twiddles(tw, twj.jobs[j], s) != cudaSuccess) return FB_FFT_ERR_CUDA;

@@ -290,23 +290,64 @@ int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long
     return FB_FFT_OK;
 }
 
+// Whether a pass of power-of-two lines (elems values) runs on the composite-radix
+// kernel instead of fft_p2.cuh's.  Small CTAs without landing buffers start and
+// drain faster, and keep more tiles in flight; the warp-specialised tiles win on
+// long lines of large passes and, up to 256 points, where input and output
+// together are about the L2 (126 MB).  us per pass, fft_p2 against this kernel,
+// contiguous lines, 2^18 / 2^21 / 2^22 / 2^23 / 2^24 / 2^26 values:
+//   64     3.5 / 7.2 / 12.1 / 21.3 / 46.0 / 182    3.3 / 5.6 /  9.9 / 21.4 / 40.9 / 154
+//   128    3.4 / 6.7 / 10.8 / 19.1 / 46.3 / 179    3.5 / 5.6 /  9.5 / 20.3 / 40.6 / 152
+//   256    3.5 / 6.6 / 10.4 / 18.2 / 45.8 / 172    3.4 / 6.0 /  8.8 / 19.3 / 41.2 / 155
+//          (2^20: 4.4 against 4.8)
+//   512    5.2 / 8.9 / 14.7 / 25.6 / 47.7 / 169    3.4 / 6.8 / 11.8 / 24.5 / 47.2 / 174
+//   1024   6.0 / 9.9 / 16.0 / 27.8 / 49.0 / 173    3.4 / 6.5 / 11.2 / 23.1 / 44.2 / 163
+//   2048   5.2 / 9.0 / 15.5 / 26.7 / 47.4 / 172    3.4 / 7.2 / 12.9 / 25.9 / 49.9 / 184
+//   4096   5.0 / 8.6 / 15.4 / 26.9 / 47.4 / 173    3.8 / 8.0 / 14.9 / 30.8 /   -  / 201
+//          (2^15: 4.2 against 3.4; 2^20: 5.5 against 6.3)
+// Strided lines: 64 x 256 grids of 2^22 / 2^24 values 25.9 / 114 against 18.5 /
+// 99 us, 128 x 256 23.8 / 102 against 20.5 / 100; 256 points and more stay (2^24:
+// 90 against 98).
+inline bool pow2_on_mr(long long L, long long elems, int io)
+{
+    const long long mib = 16 * elems >> 20;  // read and written
+    if (io == kIoCC) return L == 64 || L == 128;
+    if (io != kIoNN) return false;
+    switch (L) {
+    case 64: return mib <= 96 || mib > 192;
+    case 128: return mib <= 48 || mib > 192;
+    case 256: return (mib > 24 && mib <= 96) || mib > 192;
+    case 512: return mib <= 384;
+    case 1024: return true;
+    case 2048: return mib <= 160;
+    case 4096: return mib <= 6;
+    default: return false;
+    }
+}
+
 // Fill a line pass: L-point DFTs over lines (o, c); strides in elements.
 // `twb` receives the stage twiddle tables the pass reads: it provides
 // bool stages(L, radix, nst, off) writing the table offsets of the nst
 // stages, then (off[nst]) that of a split last stage's factor table, and
-// returns false when it has no room for them.  per_kernel: the passes of the
-// batched-uneven engine 1, whose tiles go through offset tables.
+// returns false when it has no room for them.  per_kernel keeps the lines off
+// the composite-radix kernel: the passes of the batched-uneven engine 1, whose
+// tiles go through offset tables, and allocation-free calls on powers of two,
+// whose timeout switch needs bounded waits.  route_elems: the pass size that
+// chooses the kernel when it is not the pass's own.
 template <class Twiddles>
 int make_line_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long C,
                    long long in_sn, long long in_sc, long long in_so, long long out_sk, long long out_sc,
                     long long out_so, bool in_tfast, bool out_tfast, bool ptw, bool odd_first = false,
-                   int max_lines = 0, bool tc = false, bool per_kernel = false)
+                   int max_lines = 0, bool tc = false, bool per_kernel = false, long long route_elems = 0)
 {
     const bool pow2_len = (L & (L - 1)) == 0;
     // lengths with a factor 3 or 5: the composite-radix kernel (62.6 against
     // 148.4 us on 1000-point lines x 20001, 146 against 694 us on a 120 x 150 x
-    // 144 x 4 volume forward and back); per_kernel keeps the offset-table kernels
-    if (!pow2_len && !per_kernel)
+    // 144 x 4 volume forward and back)
+    const int io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
+    const bool tc_pass = tc && pow2_len && line_kernel_p2tc(256, true, ilog2ll(L), io).fn != nullptr;
+    const bool on_mr = !pow2_len || (!tc_pass && pow2_on_mr(L, route_elems > 0 ? route_elems : O * C * L, io));
+    if (on_mr && !per_kernel)
         return make_mr_pass(p, twb, L, O, C, in_sn, in_sc, in_so, out_sk, out_sc, out_so, in_tfast, out_tfast, ptw);
     p = PassPlan{};  // zero descriptor, default member values (no offset tables)
     PassDesc& d = p.d;
@@ -328,10 +369,10 @@ int make_line_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long lo
         // Compile-time kernels: strided tiles want 16 lines for 128-byte rows,
         // so long lines on a strided side take the 512-thread kernel.
         if (in_tfast && !out_tfast) return FB_FFT_ERR_UNSUPPORTED_SIZE;  // never planned
-        p.io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
+        p.io = io;
         // radix-16 stages on the tensor cores for L >= 256: 256-thread CTAs, two per
         // SM, so one CTA's butterflies overlap the other's matrix products
-        p.tc = tc && line_kernel_p2tc(256, true, p.lg, p.io).fn != nullptr;
+        p.tc = tc_pass;
         p.threads = (!p.tc && cfast && L >= 512) ? 512 : 256;
         // short contiguous lines: 128-thread CTAs, three per SM, three tiles in flight each
         if (!p.tc && !cfast && L >= 32 && L <= 256) p.threads = nn_small_threads(L);

@@ -12,6 +12,7 @@ LineKernel line_kernel_mr_fwd_cc_a(int L)
 #define FB_MR_CASE(N) \
     case N: return mr_entry<true, N, kIoCC>();
         FB_MR_LENGTHS_A(FB_MR_CASE)
+        FB_MR_POW2_CC(FB_MR_CASE)
     default: return LineKernel{nullptr, 0, false, 0, 0};
     }
 }

@@ -12,6 +12,7 @@ LineKernel line_kernel_mr_fwd_nn_a(int L)
 #define FB_MR_CASE(N) \
     case N: return mr_entry<true, N, kIoNN>();
         FB_MR_LENGTHS_A(FB_MR_CASE)
+        FB_MR_POW2_NN(FB_MR_CASE)
     default: return LineKernel{nullptr, 0, false, 0, 0};
     }
 }

@@ -20,9 +20,10 @@
 // strided form of the same stages needed 75 instructions and 96 registers (83 us
 // on the 1000-point lines), which is why the length is a template parameter.
 // The narrow strided tiles are bound by latency and the load/store path:
-// 10^6 points x 16 266 -> 134 us.  Power-of-two lengths stay on fft_p2.cuh, whose
-// warp-specialised tiles measured faster there (4096 x 16384 173 against 201 us,
-// 2^20 x 32 209 against 243-269, 2048 x 2048 71 against 80).
+// 10^6 points x 16 266 -> 134 us.  Powers of two share the work with fft_p2.cuh
+// (pow2_on_mr in fb_plan.h says which goes where); its warp-specialised tiles stay
+// faster on 4096 x 16384 (173 against 201 us), on the four-step passes (2^20 x 32
+// 209 against 243-269) and on long strided lines.
 #pragma once
 
 #include "fft_device.cuh"

@@ -1,6 +1,7 @@
 // mr_lengths.h -- every length the composite-radix line passes are compiled
 // for: the 2^a 3^b 5^c from 3 to 4096 that are not a power of two, in two
-// halves (one translation unit each per layout and direction).
+// halves (one translation unit each per layout and direction), and the powers of
+// two whose contiguous or strided lines they take too (pow2_on_mr).
 #pragma once
 
 #define FB_MR_LENGTHS_A(K) \
@@ -15,3 +16,6 @@
     K(1600) K(1620) K(1728) K(1800) K(1875) K(1920) K(1944) K(2000) K(2025) K(2160) K(2187) K(2250) K(2304) \
     K(2400) K(2430) K(2500) K(2560) K(2592) K(2700) K(2880) K(2916) K(3000) K(3072) K(3125) K(3200) K(3240) \
     K(3375) K(3456) K(3600) K(3645) K(3750) K(3840) K(3888) K(4000) K(4050)
+
+#define FB_MR_POW2_NN(K) K(64) K(128) K(256) K(512) K(1024) K(2048) K(4096)
+#define FB_MR_POW2_CC(K) K(64) K(128)

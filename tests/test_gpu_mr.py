@@ -56,3 +56,34 @@ def test_strided_lines(fb, n):
 def test_fourstep(fb, n, direction):
     x = inputs.normal_c64((3, n), n)
     check(run(fb, x, [n], 3, direction, lead=1, scale=True), x, [n], direction, direction == 1)
+
+
+@pytest.mark.parametrize("n", [64, 128, 256, 512, 1024, 2048, 4096])
+def test_power_of_two_lines(fb, n):
+    """Powers of two below every size limit of the choice of kernel, ragged tiles."""
+    x = inputs.uniform_c64(((1 << 18) // n + 3, n), n)
+    check(run(fb, x, [n], len(x), -1, lead=1), x, [n], -1)
+    check(run(fb, x, [n], len(x), 1, scale=True, inplace=True), x, [n], 1, True)
+    if n <= 128:
+        for cols, direction in ((3, -1), (25, 1)):
+            z = inputs.normal_c64((2, n, cols), n + cols)
+            check(run(fb, z, [n, cols], 2, direction, lead=cols & 1, inplace=cols == 25), z, [n, cols], direction)
+
+
+@pytest.mark.parametrize("n,mib", [(64, 96), (128, 48), (128, 192), (256, 24), (256, 96), (256, 192), (512, 384),
+                                   (2048, 160), (4096, 6)])
+def test_power_of_two_limits(fb, n, mib):
+    """The largest batch on one side of a size limit (MiB read and written), the
+    smallest on the other, and a host-array call whose chunks lie below it."""
+    import torch
+    for batch in ((mib << 16) // n, ((mib + 1) << 16) // n):
+        x = inputs.uniform_c64((batch, n), n + batch)
+        y = run(fb, x, [n], batch, -1).reshape(batch, n)
+        i = np.r_[0:3, batch // 2, batch - 3:batch]
+        check(y[i], x[i], [n], -1)
+        hx = torch.empty(batch * n, dtype=torch.complex64, pin_memory=True)
+        hy = torch.empty(batch * n, dtype=torch.complex64, pin_memory=True)
+        hx.numpy()[:] = x.reshape(-1)
+        with fb.Plan([n], batch) as p:
+            p.exec_host(hx.numpy(), hy.numpy(), -1)
+        assert np.array_equal(hy.numpy().reshape(batch, n), y)
