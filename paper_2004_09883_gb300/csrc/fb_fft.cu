@@ -374,12 +374,14 @@ int make_uneven_pass(PassPlan& p, TwiddleBuilder& twb, long long L, long long O,
     return FB_FFT_OK;
 }
 
-// Issue cost of one tile of L-point lines with a strided side in k_fft_uneven,
+// Issue cost of one tile of T L-point lines with a strided side in k_fft_uneven,
 // in warp instructions: per stage of radix R, a butterfly is about 14 R + 30.
-long long uneven_tile_cost(const MrConfig& c)
+long long uneven_tile_cost(int L, int T)
 {
+    const MrSchedule& s = uneven_schedule(L, false);
     long long cost = 300;
-    for (int s = 0; s < c.n; ++s) cost += (c.T * (c.L / c.radix[s]) + 31) / 32 * (14LL * c.radix[s] + 30);
+    if (L == 1) return cost + 2 * ((T + 31) / 32 * 44LL);  // two copies
+    for (int k = 0; k < s.n; ++k) cost += (T * (L / s.radix[k]) + 31) / 32 * (14LL * s.radix[k] + 30);
     return cost;
 }
 
@@ -394,21 +396,23 @@ int split_uneven(long long n, long long* n1, long long* n2)
     for (long long d = 1; d * d <= n; ++d)
         if (n % d == 0 && n / d <= kUnevenMaxLen) base = d;
     if (base == 0) return FB_FFT_ERR_UNSUPPORTED_SIZE;
-    auto seg = [&](long long a) {  // shorter strided row of the pair (a, n / a)
-        const long long b = n / a;
-        return std::min(uneven_shape(a, b, kIoCCP).T, uneven_shape(b, a, kIoNC).T);
+    struct Pair {
+        int seg;         // shorter strided row
+        long long cost;  // instructions
     };
-    auto cost = [&](long long a) {
+    auto pair = [&](long long a) {  // (a, n / a)
         const long long b = n / a;
-        const MrConfig ca = uneven_shape(a, b, kIoCCP), cb = uneven_shape(b, a, kIoNC);
-        return (b + ca.T - 1) / ca.T * uneven_tile_cost(ca) + (a + cb.T - 1) / cb.T * uneven_tile_cost(cb);
+        const int ta = uneven_lines(a, b, kIoCCP), tb = uneven_lines(b, a, kIoNC);
+        return Pair{std::min(ta, tb), (b + ta - 1) / ta * uneven_tile_cost((int)a, ta) +
+                                          (a + tb - 1) / tb * uneven_tile_cost((int)b, tb)};
     };
-    const int min_seg = std::min(8, seg(base));
-    long long best = base, best_cost = cost(base);
+    const Pair first = pair(base);
+    const int min_seg = std::min(8, first.seg);
+    long long best = base, best_cost = first.cost;
     for (long long a = 1; a <= kUnevenMaxLen && a <= n; ++a) {
-        if (n % a || n / a > kUnevenMaxLen || seg(a) < min_seg) continue;
-        const long long c = cost(a);
-        if (c < best_cost) best = a, best_cost = c;
+        if ((unsigned)n % (unsigned)a || n / a > kUnevenMaxLen) continue;  // n <= kUnevenMaxLen^2
+        const Pair p = pair(a);
+        if (p.seg >= min_seg && p.cost < best_cost) best = a, best_cost = p.cost;
     }
     *n1 = best, *n2 = n / best;
     return FB_FFT_OK;

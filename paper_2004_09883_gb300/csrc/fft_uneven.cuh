@@ -609,11 +609,27 @@ inline const MrSchedule& uneven_schedule(int L, bool contiguous)
     return table.s[contiguous ? 1 : 0][L];
 }
 
-// Shape of a job of L-point lines (C per outer index) on the one-kernel
-// batched-uneven engine: the composite-radix schedule of radices up to 16, and
-// as many lines per tile as fit 4096 values -- any number of contiguous lines
-// (at most 128), a power of two where a side is strided (rows of
-// T consecutive values: 16, or 32 for short lines, whatever fits).
+// Lines per tile of a job of L-point lines (C per outer index): as many as fit
+// 4096 values -- any number of contiguous lines (at most 128), a power of two
+// where a side is strided (rows of T consecutive values: 16, or 32 for short
+// lines, whatever fits).
+inline int uneven_lines(long long L, long long C, int io)
+{
+    auto floor2 = [](long long x) {
+        long long p = 1;
+        while (p * 2 <= x) p *= 2;
+        return p;
+    };
+    long long T = std::max(1LL, kUnevenCap / L);
+    if (io == 0)  // contiguous on both sides
+        T = std::min<long long>(std::min<long long>(T, kUnevenMaxLines), C);
+    else
+        T = std::min(std::min(floor2(T), L <= 64 ? 32LL : 16LL), C <= 1 ? 1LL : 2 * floor2(C - 1));
+    return (int)std::max(1LL, T);
+}
+
+// Shape of such a job on the one-kernel batched-uneven engine: the
+// composite-radix schedule of radices up to 16, and uneven_lines per tile.
 inline MrConfig uneven_shape(long long L, long long C, int io)
 {
     MrConfig c{};
@@ -625,17 +641,7 @@ inline MrConfig uneven_shape(long long L, long long C, int io)
         c.ns[i] = ns;
         ns *= c.radix[i];
     }
-    auto floor2 = [](long long x) {
-        long long p = 1;
-        while (p * 2 <= x) p *= 2;
-        return p;
-    };
-    long long T = std::max(1LL, kUnevenCap / L);
-    if (io == 0)  // contiguous on both sides
-        T = std::min<long long>(std::min<long long>(T, kUnevenMaxLines), C);
-    else
-        T = std::min(std::min(floor2(T), L <= 64 ? 32LL : 16LL), C <= 1 ? 1LL : 2 * floor2(C - 1));
-    c.T = (int)std::max(1LL, T);
+    c.T = uneven_lines(L, C, io);
     return c;
 }
 
