@@ -407,9 +407,9 @@ int fb_fft_server_create(fb_fft_server_t* srv, int slots, long long hbm_cap_byte
  * the memory budget holds them, at most max_requests and 1024 jobs) run
  * together: their job descriptors, with each request's own addresses, go to
  * the device in one copy and run as one launch per phase and direction (at
- * most six launches for the whole batch); 1-D lengths with a four-step factor
- * above 512 points, each large enough to fill the GPU, run their plan's two
- * passes beside them, in any batch and alone.  The batch grows with the queue:
+ * most six launches for the whole batch); 1-D requests of 700,000 values
+ * (length x batch) and more with a four-step factor above 512 points run their
+ * plan's two passes before them, in any batch and alone.  The batch grows with the queue:
  * a request that finds a slot free starts at once, alone.  Results do not
  * depend on what else is in the batch (same bits alone and in any batch);
  * those of the job table can differ in the last bits from the per-request

@@ -1569,6 +1569,12 @@ int recipe_create(BatchRecipe** out, int rank, const long long* dims, long long 
         if (q.d.ntiles >= (1LL << 30)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
     BatchRecipe* r = new (std::nothrow) BatchRecipe();
     if (!r) return FB_FFT_ERR_ALLOC;
+    r->by_plan = rank == 1 && N > kUnevenMaxLen && N * batch >= kBatchPlanValues &&
+                 std::min(passes[0].d.T, passes[1].d.T) < kBatchRows;
+    if (r->by_plan) {
+        *out = r;
+        return FB_FFT_OK;
+    }
     const long long tw_elems = std::max(2LL, twb.total);
     if (cudaMalloc(&r->tw, (size_t)tw_elems * sizeof(float2)) != cudaSuccess) {
         cudaGetLastError();
@@ -1605,7 +1611,6 @@ int recipe_create(BatchRecipe** out, int rank, const long long* dims, long long 
         r->jobs.push_back(j);
         r->phases = std::max(r->phases, q.group + 1);
         r->tiles += q.d.ntiles;
-        if (q.io != kIoNN) r->rows = std::min(r->rows, q.d.T);
     }
     *out = r;
     return FB_FFT_OK;

@@ -35,6 +35,27 @@ struct BatchJob {
     bool last;        // the job that finishes the transform (takes the 1/N scale)
     size_t smem;      // shared memory its tiles need (bytes)
 };
+// A four-step request whose strided tiles would move rows of fewer values than
+// kBatchRows (64 bytes; factors above 512 points) and which has at least
+// kBatchPlanValues values (length x batch) runs its plan's two launches in a batch
+// instead of jobs: their tiles are wider or moved by the copy engine.  A smaller
+// request leaves most SMs idle in them: two dependent launches per request, one
+// request after another on the slot's stream, against a job table that runs all
+// requests' tiles together.  us per burst of 1, 4, 16 equal requests (one slot busy),
+// jobs against plan:
+//   78125    35  38  53 / 25  48 142      729000   41  68 179 / 32  73 248
+//   262440   36  43  81 / 29  65 202      10^6     45  82 263 / 34  85 293
+//   500000   38  55 126 / 29  67 239      1296000  52 103 368 / 42 109 411
+//   2^19     38  54 118 / 32  76 257      1500000  50 120 422 / 39 102 357
+//   640000   40  61 159 / 31  74 244      2^21     57 146 566 / 42 118 417
+// In mixed bursts of 128 and more several slots' launches overlap, and the plans win
+// from lower sizes on.  256 requests of a mix, six mixes, us with every such
+// length by plan 1202 on average, from 500000 values 1199, 700000 1213, 10^6 1257,
+// 1400000 1269; 16 to 64 requests are 4 to 25 % faster with the limit at 700000
+// than with every length by plan.
+constexpr int kBatchRows = 8;
+constexpr long long kBatchPlanValues = 700000;
+
 // Every job of one request shape (rank, dims, batch): up to three phases
 // (one per axis of a 2-D / 3-D shape; columns then rows of a 1-D four-step
 // length), twiddle tables in a device buffer of its own.
@@ -44,7 +65,9 @@ struct BatchRecipe {
     long long scratch_bytes = 0;  // four-step intermediate of one request
     long long table_bytes = 0;    // device bytes the recipe holds
     long long tiles = 0;          // tiles of all its jobs
-    int rows = 32;                // shortest row of values a strided tile of its jobs moves
+    // In a batch this shape's requests run their plan's own passes instead of
+    // jobs (long 1-D lengths, see kBatchRows): no jobs, no tables
+    bool by_plan = false;
     float scale = 1.f;            // 1 / (elements of one transform)
     float2* tw = nullptr;
 };

@@ -21,7 +21,7 @@
 // of such requests that fits the budget (up to max_batch), writes their jobs
 // with the requests' own addresses into the slot's pinned job table, copies
 // it to the device with one copy and runs it as one launch per phase and
-// direction (at most six); long 1-D lengths run their plan's passes beside
+// direction (at most six); long 1-D requests run their plan's passes before
 // them (kBatchRows).  Host work per request is then filling two or
 // three descriptors instead of encoding tensor maps and launching kernels;
 // the batch grows by itself with the queue, so an idle server still starts
@@ -119,23 +119,11 @@ struct ShapeKey {
 struct PlanEntry {
     fb_fft_plan_t plan = nullptr;
     host::BatchRecipe* recipe = nullptr;  // null: this shape runs per request
-    // In a batch this shape's requests run their plan's own passes instead of
-    // its recipe's jobs (long 1-D lengths, see kBatchRows)
-    bool by_plan = false;
     unsigned flags = 0;
     long long scratch = 0, io = 0, table = 0;
     long long last_use = 0;
     int users = 0;  // queued + running requests holding it
 };
-
-// Four-step jobs whose strided tiles move rows of fewer values than this (64
-// bytes; factors above 512 points) spend most of the one-kernel engine's load and
-// store path on pieces of a sector or less; such a request fills the GPU by
-// itself, and its plan's two launches, whose tiles are wider or moved by the copy
-// engine, run it faster.  256 waiting requests, 81 % of whose values are in such
-// lengths: 1637 us with none of them by plan, 1264 with rows of fewer than 4
-// values (factors above 1024), 1235 with fewer than 8.
-constexpr int kBatchRows = 8;
 
 // Jobs one slot's table holds (a batch of up to 1024 jobs: 341 four-step or
 // 3-D requests, more of the others).
@@ -240,7 +228,6 @@ int get_plan(fb_fft_server_s* s, int rank, const long long* dims, long long batc
             e.recipe = nullptr;
         }
         if (e.recipe) e.table += e.recipe->table_bytes;
-        e.by_plan = e.recipe && rank == 1 && e.recipe->rows < kBatchRows;
         // the twiddle tables are written on the build stream; requests run on
         // the slots' streams, so the tables must be complete before the first
         const cudaError_t se = cudaStreamSynchronize(s->build);
@@ -262,7 +249,7 @@ long long up_align(long long n) { return (n + kArenaAlign - 1) / kArenaAlign * k
 
 long long scratch_of(const PlanEntry* pe, bool batched)
 {
-    return batched && !pe->by_plan ? pe->recipe->scratch_bytes : pe->scratch;
+    return batched && !pe->recipe->by_plan ? pe->recipe->scratch_bytes : pe->scratch;
 }
 
 long long request_need(const PlanEntry* pe, bool host_io, bool batched)
@@ -391,7 +378,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
                 const Req& r = sl.reqs[i];
                 if ((r.direction == FB_FFT_FORWARD) != fwd) continue;
                 char* block = sl.offs[i] >= 0 ? s->arena.base + sl.offs[i] : nullptr;
-                if (r.pe->by_plan) continue;
+                if (r.pe->recipe->by_plan) continue;
                 const long long scr = up_align(r.pe->recipe->scratch_bytes);
                 // host arrays: the transform runs in place in the staging buffer
                 const float2* in = r.host_io ? reinterpret_cast<const float2*>(block + scr)
@@ -433,7 +420,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
     }
     for (size_t i = 0; i < sl.reqs.size(); ++i) {
         const Req& r = sl.reqs[i];
-        if (!r.pe->by_plan) continue;
+        if (!r.pe->recipe->by_plan) continue;
         char* block = sl.offs[i] >= 0 ? s->arena.base + sl.offs[i] : nullptr;
         char* stage = block + up_align(scratch_of(r.pe, true));
         const int rc = host::plan_exec_on(r.pe->plan, r.host_io ? stage : r.in, r.host_io ? stage : r.out, r.direction,
