@@ -96,6 +96,12 @@ struct PassDesc {
     // k 2^in_tl + n mod 2^in_tl).
     int in_tl;
     int out_blk;  // four-step columns: 1 = write such blocks
+    // Composite-radix strided lines, > 0: an outer index has only `fold` lines and a
+    // tile takes those of several (line t: outer index t / fold, column t % fold;
+    // fold_mag = ceil(2^16 / fold); in_so / out_so lie between outer indices, the
+    // tile starts at line c0 in_sc)
+    int fold;
+    unsigned fold_mag;
     // k_fft_uneven: multiply-high reciprocal of L / radix[s] (0 when that is
     // 1), the exchange buffer stage s reads (row stride, extra values after
     // every block of ns[s], step between a butterfly's inputs: MrConfig),

@@ -41,6 +41,14 @@ inline int nn_small_threads(long long L)
 // Contiguous composite-radix tiles hold fewer lines where a pass would
 // otherwise have fewer tiles than this many per SM of a GB300.
 constexpr int kMrMinTilesPerSm = 2, kMrSms = 152;
+// Strided tiles take the lines of several outer indices while this many tiles are
+// left: one per SM, or, where a CTA has an SM to itself (MrConfig::in_place), a
+// quarter of that: a few full tiles beat many nearly empty ones in several waves.
+// 1026 small grids against the older kernels, limits of 304 / 152 / 76 / 38 tiles for
+// all: geometric mean 0.704 / 0.691 / 0.684 / 0.684, more than 3 % slower 48 / 29 / 12 /
+// 2; below 152 the small tiles lose up to a tenth to unfolded ones (160 x 2 x 640 22.1
+// us unfolded, 22.6 / 24.6 with limits of 152 / 38).
+constexpr int kMrFoldTiles = kMrSms, kMrFoldTilesInPlace = kMrSms / 4;
 
 enum BufKind { kBufIn = 0, kBufOut = 1, kBufScratch = 2 };
 constexpr size_t kMaxSmemBytes = 227 * 1024;
@@ -259,8 +267,26 @@ int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long
     for (int s = 0; s < d.nst; ++s) d.twoff[s] = off[s];
     // fewer lines per tile than the kernel's most when that leaves SMs idle
     // (contiguous lines: the kernel takes any number up to c.T)
-    const long long T =
+    long long T =
         p.io != kIoNN ? c.T : std::max(1LL, std::min<long long>(c.T, C / (kMrMinTilesPerSm * kMrSms)));
+    // Strided lines with a short trailing extent: a tile of C <= T / 2 lines would
+    // leave most of its threads idle, so it takes those of as many outer indices as
+    // fit, while enough tiles are left (kMrFoldTiles).  us per pass of 2^21 values: the older
+    // kernels, whose tile width followed C / tiles of one outer index / this:
+    //   125 x 2  69 / 94 / 20      250 x 2  47 / 69 / 18      480 x 2  30 / 47 / 14
+    //   250 x 4  30 / 38 / 16      540 x 2  43 / 71 / 18     1000 x 2  26 / 37 / 14
+    // (tiles of one outer index were the faster only where 25-point radices and
+    // copy-engine tiles were not involved: 243 x 2 55 / 51 / 14, 120 x 3 59 / 24 / 12).
+    if (p.io == kIoCC && C > 0 && in_so % C == 0 && out_so % C == 0) {
+        const long long k = std::min<long long>(c.T / C, O / (c.in_place ? kMrFoldTilesInPlace : kMrFoldTiles));
+        if (k >= 2) {
+            d.fold = (int)C;
+            d.fold_mag = (unsigned)((65536 + C - 1) / C);
+            in_sc = in_so / C, out_sc = out_so / C;
+            T = k * C;
+            C *= O, O = 1;
+        }
+    }
     p.threads = c.threads;
     d.T = (int)T;
     d.logT = ilog2ll(T);
@@ -280,7 +306,7 @@ int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long
         if (L % b == 0 && (b == L || (b * T * 8) % 128 == 0)) br = b;
     const bool in_ok = !in_tfast || (T % 2 == 0 && in_sn % 2 == 0 && (O == 1 || in_so % 2 == 0));
     const bool out_ok = !out_tfast || (T % 2 == 0 && out_sk % 2 == 0 && (O == 1 || out_so % 2 == 0));
-    p.async_ok = c.in_place && br > 0 && in_ok && out_ok && C < (1LL << 31) && O < (1LL << 31);
+    p.async_ok = c.in_place && !d.fold && br > 0 && in_ok && out_ok && C < (1LL << 31) && O < (1LL << 31);
     d.box_rows = br > 0 ? br : 1;
     d.tpo_mag = (d.tiles_per_o > 1 && d.ntiles < (1LL << 32))
                     ? (unsigned)(((1ULL << 32) + d.tiles_per_o - 1) / d.tiles_per_o) : 0u;

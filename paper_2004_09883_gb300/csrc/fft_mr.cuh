@@ -173,6 +173,15 @@ __device__ __forceinline__ float2 mr_ptw(const PassDesc& d, unsigned m)
     return cmul(__ldg(d.ptw_hi + (m >> d.ptw_log)), __ldg(d.ptw_lo + (m & ((1u << d.ptw_log) - 1))));
 }
 
+// Where line t of a strided tile starts relative to its first line (so: values
+// between outer indices).
+__device__ __forceinline__ long long mr_line(const PassDesc& d, int t, long long so)
+{
+    if (d.fold == 0) return t;
+    const int o = (int)((unsigned)t * d.fold_mag >> 16);
+    return o * so + (t - o * d.fold);
+}
+
 template <int L, int IO>
 struct Mr {
     static constexpr MrConfig c = mr_config(L, IO);
@@ -231,7 +240,8 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u][r] = p[r * LR * C.T];
             } else if constexpr (first) {
-                const float2* p = IN_T ? gin + (long long)j[u] * d.in_sn + t[u] : gin + t[u] * L + j[u];
+                const float2* p = IN_T ? gin + (long long)j[u] * d.in_sn + (IO == 1 ? mr_line(d, t[u], d.in_so) : t[u])
+                                       : gin + t[u] * L + j[u];
                 long long step = IN_T ? LR * d.in_sn : LR;
                 if constexpr (IO == 2) {
                     if (d.in_tl) {
@@ -266,7 +276,8 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
                 for (int r = 0; r < R; ++r) p[r * Ns] = v[u][r];
             } else {
                 // Ns = L / R: the outputs of butterfly j are j + r Ns
-                float2* p = OUT_T ? gout + (long long)j[u] * d.out_sk + t[u] : gout + t[u] * L + j[u];
+                float2* p = OUT_T ? gout + (long long)j[u] * d.out_sk + (IO == 1 ? mr_line(d, t[u], d.out_so) : t[u])
+                                  : gout + t[u] * L + j[u];
                 const long long step = OUT_T ? Ns * d.out_sk : Ns;
                 if constexpr (IO == 3) {
                     // exp(-2 pi i c (j + r Ns) / N): products of the tile's own factors
