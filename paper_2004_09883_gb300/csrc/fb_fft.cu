@@ -238,7 +238,7 @@ struct fb_fft_plan_s {
         long long tiles = 0;
         long long grid = 0;
         size_t smem = 0;
-        PassDesc* d_jobs = nullptr;
+        UnevenDesc* d_jobs = nullptr;
         int* d_tiles = nullptr;
     };
     UnevenPhase uphase[2];
@@ -332,7 +332,7 @@ int make_uneven_pass(PassPlan& p, TwiddleBuilder& twb, long long L, long long O,
                      bool in_tfast, bool out_tfast, bool ptw)
 {
     p = PassPlan{};
-    PassDesc& d = p.d;
+    UnevenDesc& d = p.d;
     if (L < 1 || L > kUnevenMaxLen || !is_smooth(L)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
     p.kind = 4;
     p.io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
@@ -976,7 +976,7 @@ int build_plan(fb_fft_plan_s* p)
             // place of the exec's pointers, and tile prefixes -- each phase's,
             // and both phases' for the one-launch form -- and that form's
             // counters, in one device allocation
-            std::vector<PassDesc> jobs;
+            std::vector<UnevenDesc> jobs;
             std::vector<int> tiles;
             fb_fft_plan_s::UnevenPhase* tabs[3] = {&p->uphase[0], &p->uphase[1], &p->uone};
             size_t job_at[3], tile_at[3];
@@ -987,7 +987,7 @@ int build_plan(fb_fft_plan_s* p)
                 long long t = 0;
                 for (int i : u.jobs) {
                     const PassPlan& q = p->passes[i];
-                    PassDesc d = q.d;
+                    UnevenDesc d = q.d;
                     d.in = reinterpret_cast<const float2*>(static_cast<uintptr_t>(q.src_off));
                     d.in_buf = q.src == kBufIn ? 0 : (q.src == kBufOut ? 1 : 2);
                     d.out = reinterpret_cast<float2*>(static_cast<uintptr_t>(q.dst_off));
@@ -1001,7 +1001,7 @@ int build_plan(fb_fft_plan_s* p)
                 if (t >= (1LL << 31)) return FB_FFT_ERR_UNSUPPORTED_SIZE;
                 tiles.push_back((int)t);
             }
-            const size_t jb = jobs.size() * sizeof(PassDesc), tb = tiles.size() * sizeof(int);
+            const size_t jb = jobs.size() * sizeof(UnevenDesc), tb = tiles.size() * sizeof(int);
             const size_t sb_at = (jb + tb + 15) & ~(size_t)15;
             const int nsync = 3 + p->uneven_slots;
             const size_t sb = (size_t)nsync * sizeof(unsigned long long);
@@ -1010,7 +1010,7 @@ int build_plan(fb_fft_plan_s* p)
                 p->d_uneven = nullptr;
                 return FB_FFT_ERR_ALLOC;
             }
-            PassDesc* dj = static_cast<PassDesc*>(p->d_uneven);
+            UnevenDesc* dj = static_cast<UnevenDesc*>(p->d_uneven);
             int* dt = reinterpret_cast<int*>(static_cast<char*>(p->d_uneven) + jb);
             p->d_sync = reinterpret_cast<unsigned long long*>(static_cast<char*>(p->d_uneven) + sb_at);
             if (jb) FB_CK(cudaMemcpyAsync(dj, jobs.data(), jb, cudaMemcpyHostToDevice, p->stream));
@@ -1649,7 +1649,7 @@ int uneven_resident(bool forward, size_t smem, bool inl, long long* cap)
     return FB_FFT_OK;
 }
 
-int batch_launch(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
+int batch_launch(bool forward, const UnevenDesc* jobs, const int* tile_start, int njobs, long long tiles,
                  size_t smem, cudaStream_t stream)
 {
     if (njobs <= 0 || tiles <= 0) return FB_FFT_OK;
@@ -1671,7 +1671,7 @@ int batch_launch(bool forward, const PassDesc* jobs, const int* tile_start, int 
     return FB_FFT_OK;
 }
 
-int batch_launch_inline(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
+int batch_launch_inline(bool forward, const UnevenDesc* jobs, const int* tile_start, int njobs, long long tiles,
                         size_t smem, cudaStream_t stream)
 {
     if (njobs <= 0 || tiles <= 0) return FB_FFT_OK;
@@ -1684,7 +1684,7 @@ int batch_launch_inline(bool forward, const PassDesc* jobs, const int* tile_star
     std::memset(&p, 0, sizeof(p));
     p.a.njobs = njobs;
     p.a.scale_on = 1;
-    std::memcpy(p.jobs, jobs, (size_t)njobs * sizeof(PassDesc));
+    std::memcpy(p.jobs, jobs, (size_t)njobs * sizeof(UnevenDesc));
     std::memcpy(p.tile_start, tile_start, (size_t)(njobs + 1) * sizeof(int));
     const cudaError_t e = uneven_launch_inline(forward, p, std::min(tiles, cap), smem, stream);
     if (e != cudaSuccess) return cuda_fail(e, "k_fft_uneven_inline (server batch)");

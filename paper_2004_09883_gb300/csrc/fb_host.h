@@ -29,7 +29,7 @@ void plan_free(fb_fft_plan_t p);
 // One job of a request shape on the one-kernel engine (k_fft_uneven): its
 // descriptor with the twiddle pointers bound, and where it reads and writes.
 struct BatchJob {
-    PassDesc d;       // in / out: element offsets into the buffers src / dst name
+    UnevenDesc d;       // in / out: element offsets into the buffers src / dst name
     int phase;        // launch it runs in: jobs of phase k + 1 read what phase k wrote
     int src, dst;     // 0 the request's input, 1 its output, 2 its scratch
     bool last;        // the job that finishes the transform (takes the 1/N scale)
@@ -78,11 +78,11 @@ int recipe_create(BatchRecipe** out, int rank, const long long* dims, long long 
 void recipe_free(BatchRecipe* r);
 // One launch of k_fft_uneven over the job and tile-prefix tables in device
 // memory (njobs jobs, `tiles` tiles in all); the launch counter counts it.
-int batch_launch(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
+int batch_launch(bool forward, const UnevenDesc* jobs, const int* tile_start, int njobs, long long tiles,
                  size_t smem, cudaStream_t stream);
 // The same launch with the tables (host memory, at most 16 jobs) copied
 // into the kernel parameter: nothing to copy to the device beforehand.
-int batch_launch_inline(bool forward, const PassDesc* jobs, const int* tile_start, int njobs, long long tiles,
+int batch_launch_inline(bool forward, const UnevenDesc* jobs, const int* tile_start, int njobs, long long tiles,
                         size_t smem, cudaStream_t stream);
 // Record a failed CUDA call for fb_fft_last_error and map it to a status.
 int fail(cudaError_t e, const char* what);

@@ -72,19 +72,6 @@ struct PassDesc {
     // Contiguous layouts index them by line, strided ones by outer index.
     const long long* off_in;
     const long long* off_out;
-    // Batched-uneven job tables (k_fft_uneven): which exec buffer `in` and
-    // `out` refer to (0 the caller's input, 1 its output, 2 the plan's
-    // scratch; the pointer fields then hold element offsets into it), or 3:
-    // the pointer fields are the addresses themselves.
-    int in_buf;
-    int out_buf;
-    // Batched uneven lengths in one launch (k_fft_uneven_one): dependency
-    // slot s + 1 whose finished-tile counter this job's tiles raise (four-step
-    // columns), or that it waits for (four-step rows) until the counter
-    // reaches dep_need; 0 = none.
-    int dep_post;
-    int dep;
-    int dep_need;
     // Composite-radix kernels (fft_mr.cuh): lines per tile, and
     // ceil(2^32 / tiles_per_o) where that divides a tile number below 2^32
     // (0: one outer index, or 64-bit numbers).
@@ -102,7 +89,27 @@ struct PassDesc {
     // tile starts at line c0 in_sc)
     int fold;
     unsigned fold_mag;
-    // k_fft_uneven: multiply-high reciprocal of L / radix[s] (0 when that is
+};
+
+// A job of the batched-uneven kernel (fft_uneven.cuh): a pass and what only that
+// kernel reads.  Kept apart because the merged launches of the mixed kernel carry
+// up to 64 descriptors in their parameter and copy one per tile (16 to 64 lengths 4 %
+// slower with these fields among the others).
+struct UnevenDesc : PassDesc {
+    // Job tables: which exec buffer `in` and
+    // `out` refer to (0 the caller's input, 1 its output, 2 the plan's
+    // scratch; the pointer fields then hold element offsets into it), or 3:
+    // the pointer fields are the addresses themselves.
+    int in_buf;
+    int out_buf;
+    // Batched uneven lengths in one launch (k_fft_uneven_one): dependency
+    // slot s + 1 whose finished-tile counter this job's tiles raise (four-step
+    // columns), or that it waits for (four-step rows) until the counter
+    // reaches dep_need; 0 = none.
+    int dep_post;
+    int dep;
+    int dep_need;
+    // Multiply-high reciprocal of L / radix[s] (0 when that is
     // 1), the exchange buffer stage s reads (row stride, extra values after
     // every block of ns[s], step between a butterfly's inputs: MrConfig),
     // where the second buffer and the tile's four-step factors start.

@@ -54,7 +54,7 @@ enum BufKind { kBufIn = 0, kBufOut = 1, kBufScratch = 2 };
 constexpr size_t kMaxSmemBytes = 227 * 1024;
 
 struct PassPlan {
-    PassDesc d;
+    UnevenDesc d;  // (a PassDesc to every kernel but the batched-uneven one)
     int threads;  // CTA size of the chosen kernel
     int lg;       // log2(L) for a compile-time power-of-two kernel, 0 = generic kernel
     int io;       // IoMode of the power-of-two kernel

@@ -130,7 +130,7 @@ struct PlanEntry {
 constexpr int kBatchJobs = 1024;
 constexpr int kBatchGroups = 6;  // launches per batch: three phases x two directions
 constexpr size_t kTableBytes =
-    ((kBatchJobs * sizeof(PassDesc) + (kBatchJobs + kBatchGroups) * sizeof(int)) + 255) / 256 * 256;
+    ((kBatchJobs * sizeof(UnevenDesc) + (kBatchJobs + kBatchGroups) * sizeof(int)) + 255) / 256 * 256;
 
 struct Req {
     long long tag = 0;
@@ -348,7 +348,7 @@ int start(fb_fft_server_s* s, Slot& sl, const Req& r, long long off)
 // jobs are written, then moved right behind the last job.
 int* tile_scratch_of(Slot& sl)
 {
-    return reinterpret_cast<int*>(sl.tab_host + kBatchJobs * sizeof(PassDesc));
+    return reinterpret_cast<int*>(sl.tab_host + kBatchJobs * sizeof(UnevenDesc));
 }
 
 // Put the batch on slot sl: its job table (every request's jobs with their
@@ -359,7 +359,7 @@ int* tile_scratch_of(Slot& sl)
 int start_batch(fb_fft_server_s* s, Slot& sl)
 {
     // jobs first; the tile prefixes go right behind the last job (one copy)
-    PassDesc* jobs = reinterpret_cast<PassDesc*>(sl.tab_host);
+    UnevenDesc* jobs = reinterpret_cast<UnevenDesc*>(sl.tab_host);
     int* tiles = tile_scratch_of(sl);
     struct Group {
         bool fwd;
@@ -388,7 +388,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
                 const bool scale = !fwd && (r.pe->flags & FB_FFT_SCALE_INV_N);
                 for (const host::BatchJob& j : r.pe->recipe->jobs) {
                     if (j.phase != ph) continue;
-                    PassDesc& d = jobs[nj];
+                    UnevenDesc& d = jobs[nj];
                     d = j.d;
                     d.in = j.src == 0 ? in : (j.src == 1 ? out : scratch);
                     d.out = j.dst == 1 ? out : scratch;
@@ -427,17 +427,17 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
                                           sl.stream, block, sl.err_dev);
         if (rc != FB_FFT_OK) return rc;
     }
-    int* packed_tiles = reinterpret_cast<int*>(sl.tab_host + (size_t)nj * sizeof(PassDesc));
+    int* packed_tiles = reinterpret_cast<int*>(sl.tab_host + (size_t)nj * sizeof(UnevenDesc));
     std::memmove(packed_tiles, tiles, (size_t)nt * sizeof(int));
     // groups of few jobs carry their tables in the kernel parameter; the
     // table goes to the device only for a larger group
     bool copy = false;
     for (int k = 0; k < ng; ++k) copy = copy || groups[k].njobs > kUnevenInlineJobs;
     if (copy)
-        SV_CK(cudaMemcpyAsync(sl.tab_dev, sl.tab_host, (size_t)nj * sizeof(PassDesc) + (size_t)nt * sizeof(int),
+        SV_CK(cudaMemcpyAsync(sl.tab_dev, sl.tab_host, (size_t)nj * sizeof(UnevenDesc) + (size_t)nt * sizeof(int),
                               cudaMemcpyHostToDevice, sl.stream));
-    const PassDesc* djobs = reinterpret_cast<const PassDesc*>(sl.tab_dev);
-    const int* dtiles = reinterpret_cast<const int*>(sl.tab_dev + (size_t)nj * sizeof(PassDesc));
+    const UnevenDesc* djobs = reinterpret_cast<const UnevenDesc*>(sl.tab_dev);
+    const int* dtiles = reinterpret_cast<const int*>(sl.tab_dev + (size_t)nj * sizeof(UnevenDesc));
     for (int k = 0; k < ng; ++k) {
         const Group& g = groups[k];
         const int rc = g.njobs <= kUnevenInlineJobs

@@ -5,7 +5,7 @@
 // columns; phase 1: rows); k_fft_uneven_one (below) runs both phases in ONE
 // launch, each row chunk after its columns.
 //
-// Jobs (one PassDesc per length group or four-step chunk, each with its own
+// Jobs (one UnevenDesc per length group or four-step chunk, each with its own
 // offset tables, strides, radix schedule and twiddle tables) sit in a device
 // table; a device prefix table gives each job's first global tile.
 // k_fft_uneven's persistent CTAs walk the global tiles blockIdx.x,
@@ -48,7 +48,7 @@ constexpr int kUnevenMaxLines = 128;  // contiguous lines per tile
 // and the buffers of this exec.  A job's `in` / `out` fields hold element
 // offsets into the buffer its in_buf / out_buf names, or (kind 3) addresses.
 struct UnevenArgs {
-    const PassDesc* jobs;   // [njobs]
+    const UnevenDesc* jobs;   // [njobs]
     const int* tile_start;  // [njobs + 1]: first global tile of each job; [njobs] = all tiles
     const float2* in;       // buffer 0: the caller's input
     float2* out;            // buffer 1: the caller's output
@@ -57,7 +57,7 @@ struct UnevenArgs {
     int scale_on;           // 1: jobs marked apply_scale multiply by their `scale`
     // One-launch form (k_fft_uneven_one) only: device counters, nsync of
     // them, zero between execs -- [0] tiles claimed, [1] CTAs finished,
-    // [1 + s] finished tiles of dependency slot s >= 1 (PassDesc::dep_post /
+    // [1 + s] finished tiles of dependency slot s >= 1 (UnevenDesc::dep_post /
     // dep), [nsync - 1] finished column tiles of the batch.
     unsigned long long* sync;
     int nsync;
@@ -66,11 +66,11 @@ struct UnevenArgs {
 };
 
 // Kernel argument of the inline form: the tables themselves (a.jobs and
-// a.tile_start unused).  About 5.8 KB, well under the 32 KB parameter limit.
+// a.tile_start unused).  About 7.6 KB, well under the 32 KB parameter limit.
 constexpr int kUnevenInlineJobs = 16;
 struct UnevenInlineArgs {
     UnevenArgs a;
-    PassDesc jobs[kUnevenInlineJobs];
+    UnevenDesc jobs[kUnevenInlineJobs];
     int tile_start[kUnevenInlineJobs + 1];
 };
 
@@ -81,7 +81,7 @@ struct UnevenInlineArgs {
 struct UTileIdx {
     int o, c0, Tv;
 };
-__device__ __forceinline__ UTileIdx utile_index(const PassDesc& d, int tile)
+__device__ __forceinline__ UTileIdx utile_index(const UnevenDesc& d, int tile)
 {
     UTileIdx ti;
     const int tpo = (int)d.tiles_per_o;
@@ -94,26 +94,26 @@ __device__ __forceinline__ UTileIdx utile_index(const PassDesc& d, int tile)
 
 // A job's input / output base in this exec's buffers; kind 3: the field is
 // the address itself (jobs of different requests in one server launch).
-__device__ __forceinline__ const float2* ubuf_in(const UnevenArgs& a, const PassDesc& d)
+__device__ __forceinline__ const float2* ubuf_in(const UnevenArgs& a, const UnevenDesc& d)
 {
     if (d.in_buf == 3) return d.in;
     const float2* b = d.in_buf == 0 ? a.in : (d.in_buf == 1 ? a.out : a.scratch);
     return b + (long long)reinterpret_cast<uintptr_t>(d.in);
 }
-__device__ __forceinline__ float2* ubuf_out(const UnevenArgs& a, const PassDesc& d)
+__device__ __forceinline__ float2* ubuf_out(const UnevenArgs& a, const UnevenDesc& d)
 {
     if (d.out_buf == 3) return d.out;
     float2* b = d.out_buf == 1 ? a.out : a.scratch;
     return b + (long long)reinterpret_cast<uintptr_t>(d.out);
 }
 // Global start of line (o, c) of the input / output (offset tables or strides).
-__device__ __forceinline__ const float2* uline_in(const UnevenArgs& a, const PassDesc& d, int o, int c)
+__device__ __forceinline__ const float2* uline_in(const UnevenArgs& a, const UnevenDesc& d, int o, int c)
 {
     const float2* in = ubuf_in(a, d);
     if (d.off_in) return in + (d.in_tfast ? d.off_in[o] + c : d.off_in[c]);
     return in + (long long)o * d.in_so + (long long)c * d.in_sc;
 }
-__device__ __forceinline__ float2* uline_out(const UnevenArgs& a, const PassDesc& d, int o, int c)
+__device__ __forceinline__ float2* uline_out(const UnevenArgs& a, const UnevenDesc& d, int o, int c)
 {
     float2* out = ubuf_out(a, d);
     if (d.off_out) return out + (d.out_tfast ? d.off_out[o] + c : d.off_out[c]);
@@ -139,7 +139,7 @@ struct UTile {
 };
 
 // exp(-2 pi i m / N) from the job's two split four-step tables (m < N < 2^31).
-__device__ __forceinline__ float2 uptw(const PassDesc& d, unsigned m)
+__device__ __forceinline__ float2 uptw(const UnevenDesc& d, unsigned m)
 {
     return cmul(__ldg(d.ptw_hi + (m >> d.ptw_log)), __ldg(d.ptw_lo + (m & ((1u << d.ptw_log) - 1))));
 }
@@ -189,7 +189,7 @@ __device__ __forceinline__ void usync() { asm volatile("bar.sync 1, %0;" ::"n"(k
 // (st - 1) & 1, every stage but the last writes buffer st & 1, the last stores
 // to global memory with the four-step twiddle and the scale applied.
 template <int R, bool FWD, int POS>
-__device__ __forceinline__ void ustage(const UnevenArgs& a, const PassDesc& d, const UTile& tl, int st, float2* buf)
+__device__ __forceinline__ void ustage(const UnevenArgs& a, const UnevenDesc& d, const UTile& tl, int st, float2* buf)
 {
     constexpr bool first = POS == kPosFirst;
     constexpr bool last = POS == kPosLast;
@@ -290,7 +290,7 @@ __device__ __forceinline__ void ustage(const UnevenArgs& a, const PassDesc& d, c
 
 // Stage st, any radix of a schedule.
 template <bool FWD, int POS>
-__device__ __forceinline__ void ustage_any(const UnevenArgs& a, const PassDesc& d, const UTile& tl, int st, float2* buf)
+__device__ __forceinline__ void ustage_any(const UnevenArgs& a, const UnevenDesc& d, const UTile& tl, int st, float2* buf)
 {
     switch (d.radix[st]) {
 #define FB_USTAGE(R) \
@@ -314,7 +314,7 @@ __device__ __forceinline__ void ustage_any(const UnevenArgs& a, const PassDesc& 
 }
 // Every stage of tile tl of job d, by the compute warps.
 template <bool FWD>
-__device__ __forceinline__ void utile_run(const UnevenArgs& a, const PassDesc& d, const UTile& tl, float2* buf)
+__device__ __forceinline__ void utile_run(const UnevenArgs& a, const UnevenDesc& d, const UTile& tl, float2* buf)
 {
     ustage_any<FWD, kPosFirst>(a, d, tl, 0, buf);
     if (d.ptw) {  // four-step columns: the factors of the tile's lines the last stage needs
@@ -330,7 +330,7 @@ __device__ __forceinline__ void utile_run(const UnevenArgs& a, const PassDesc& d
 
 // Control warp: ask L2 for the values a tile will read.
 __device__ __forceinline__ void uprefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-__device__ __forceinline__ void utile_prefetch(const PassDesc& d, const UTile& tl, int lane)
+__device__ __forceinline__ void utile_prefetch(const UnevenDesc& d, const UTile& tl, int lane)
 {
     const int Tv = tl.ti.Tv;
     if (d.in_tfast) {
@@ -348,7 +348,7 @@ __device__ __forceinline__ void utile_prefetch(const PassDesc& d, const UTile& t
     }
 }
 // Control warp: fill in the tile of job d.
-__device__ __forceinline__ void utile_find(const UnevenArgs& a, const PassDesc& d, int number, UTile& tl, int lane)
+__device__ __forceinline__ void utile_find(const UnevenArgs& a, const UnevenDesc& d, int number, UTile& tl, int lane)
 {
     const UTileIdx ti = utile_index(d, number);
     const bool in_c = !d.in_tfast, out_c = !d.out_tfast;
@@ -457,11 +457,11 @@ __device__ __forceinline__ void udeps_wait(const UnevenArgs& a, int dep, int nee
 }
 
 template <bool FWD, bool INL, bool ONE>
-__device__ __forceinline__ void uneven_body(const UnevenArgs& a, const PassDesc* jobs, const int* tile_start)
+__device__ __forceinline__ void uneven_body(const UnevenArgs& a, const UnevenDesc* jobs, const int* tile_start)
 {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
     float2* buf = reinterpret_cast<float2*>(smem_dyn);
-    __shared__ PassDesc sd[2];  // the descriptors of two tiles in turn
+    __shared__ UnevenDesc sd[2];  // the descriptors of two tiles in turn
     __shared__ UTile s_tile[2];
     pdl_start();
     if (threadIdx.x < kUnevenThreads) {
@@ -499,7 +499,7 @@ __device__ __forceinline__ void uneven_body(const UnevenArgs& a, const PassDesc*
             }
             const int* src = reinterpret_cast<const int*>(jobs + j);
             int* dst = reinterpret_cast<int*>(&sd[b]);
-            for (int w = lane; w < (int)(sizeof(PassDesc) / 4); w += 32) dst[w] = utab<INL>(src + w);
+            for (int w = lane; w < (int)(sizeof(UnevenDesc) / 4); w += 32) dst[w] = utab<INL>(src + w);
             __syncwarp();
             utile_find(a, sd[b], g - utab<INL>(tile_start + j), s_tile[b], lane);
             next_post = sd[b].dep_post;
