@@ -926,7 +926,9 @@ int build_plan(fb_fft_plan_s* p)
             q.d.tw = p->tw;
             continue;
         }
-        if (q.kind == 5) {  // one tile per CTA: no cap
+        if (q.kind == 5) {  // one tile per CTA: no cap; the forward kernel loads and is checked here as the others are
+            FB_CK(line_occupancy(k, q.smem, &occ));
+            if (occ < 1) return cuda_fail(cudaErrorInvalidConfiguration, "line pass occupancy");
             q.d.err = p->err;
             q.d.tw = p->tw;
             if (q.d.ptw) {
