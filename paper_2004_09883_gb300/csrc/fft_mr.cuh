@@ -167,6 +167,21 @@ __device__ __forceinline__ unsigned long long l2_evict_normal_policy()
     return pol;
 }
 
+// Wait for the tile's copies, at most kWaitLimitNs.  One tile per CTA and no cap
+// on the grid: once a CTA of the launch has given up (error word), a wait longer
+// than any copy takes ends too, or a launch of thousands of tiles whose copies
+// cannot arrive would wait the limit once per wave of CTAs.
+__device__ __forceinline__ bool mr_wait(unsigned long long* bar, unsigned parity, const int* err)
+{
+    if (mbar_try_wait(bar, parity)) return true;
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try_wait(bar, parity)) {
+        const unsigned long long t = global_ns() - t0;
+        if (t > kWaitLimitNs || (t > 1000000ULL && *static_cast<const volatile int*>(err) != 0)) return false;
+    }
+    return true;
+}
+
 // exp(-2 pi i m / N) from the split four-step tables (m < N < 2^31).
 __device__ __forceinline__ float2 mr_ptw(const PassDesc& d, unsigned m)
 {
@@ -379,12 +394,16 @@ __global__ void __maxnreg__((Mr<L, IO>::c.regs)) k_fft_mr(const __grid_constant_
                     for (int n0 = 0; n0 < L; n0 += d.box_rows)
                         tma_load_3d(buf0 + n0 * C.T, &a.tm_in, (int)c0, n0, (int)o, bar, d.err, true, pin);
                 }
-                const bool bad = !mbar_wait_bounded(bar, phase);
-                phase ^= 1u;
+                const bool bad = !mr_wait(bar, phase, d.err);
                 if (__syncthreads_or(bad)) {
-                    if (threadIdx.x == 0) atomicExch(d.err, 1);
+                    if (threadIdx.x == 0) {
+                        atomicExch(d.err, 1);
+                        bulk_wait_all();
+                        mr_wait(bar, phase, d.err);  // the tile's loads, once more, while its shared memory lives
+                    }
                     return;
                 }
+                phase ^= 1u;
             }
         }
         if (C.in_place && copied)
