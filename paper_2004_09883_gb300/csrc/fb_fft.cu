@@ -325,6 +325,29 @@ bool use_uneven_engine(int count, const long long* lengths, const fb_fft_many_op
     return true;
 }
 
+// The tiles of a job of shape c (O outer indices, d.C lines each): its exchange
+// buffers' places and tile counts, in the descriptor.  Returns the shared memory its
+// tiles need (bytes).
+size_t uneven_tiles(UnevenDesc& d, MrConfig c, long long O)
+{
+    mr_place(c);
+    for (int s = 0; s < c.n; ++s) {
+        const int lr = c.L / c.radix[s];
+        d.lr_mag[s] = lr > 1 ? (unsigned)(((1ULL << 32) + lr - 1) / lr) : 0u;
+        if (s == 0) continue;
+        d.xrow[s] = c.row[s];
+        d.xpad[s] = c.pad[s];
+        d.xstep[s] = lr + lr / c.ns[s] * c.pad[s];
+    }
+    d.xbuf = c.buf[0];
+    d.ptw_at = c.buf[0] + c.buf[1];
+    d.T = c.T;
+    d.logT = ilog2ll(c.T);
+    d.tiles_per_o = (d.C + c.T - 1) / c.T;
+    d.ntiles = O * d.tiles_per_o;
+    return (size_t)(c.buf[0] + c.buf[1] + c.ptw) * sizeof(float2);
+}
+
 // One job of the one-kernel engine: L-point DFTs over lines (o, c), strides in
 // elements (offsets into the exec buffers are set by the caller).
 int make_uneven_pass(PassPlan& p, TwiddleBuilder& twb, long long L, long long O, long long C, long long in_sn,
@@ -337,39 +360,23 @@ int make_uneven_pass(PassPlan& p, TwiddleBuilder& twb, long long L, long long O,
     p.kind = 4;
     p.io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
     p.threads = kUnevenThreads;
-    MrConfig c = uneven_shape(L, C, p.io);
+    const MrConfig c = uneven_shape(L, C, p.io);
     if (c.n < 2) return FB_FFT_ERR_UNSUPPORTED_SIZE;
-    mr_place(c);
     d.nst = c.n;
     for (int s = 0; s < c.n; ++s) d.radix[s] = c.radix[s];
     set_stage_products(d);
     const std::vector<int> off = twb.add_stages(L, d.radix, d.nst);
-    for (int s = 0; s < d.nst; ++s) {
-        const int lr = (int)L / c.radix[s];
-        d.twoff[s] = off[s];
-        d.lr_mag[s] = lr > 1 ? (unsigned)(((1ULL << 32) + lr - 1) / lr) : 0u;
-        if (s == 0) continue;
-        d.xrow[s] = c.row[s];
-        d.xpad[s] = c.pad[s];
-        d.xstep[s] = lr + lr / c.ns[s] * c.pad[s];
-    }
-    d.xbuf = c.buf[0];
-    d.ptw_at = c.buf[0] + c.buf[1];
-    const long long T = c.T;
+    for (int s = 0; s < d.nst; ++s) d.twoff[s] = off[s];
     d.L = (int)L;
-    d.T = (int)T;
-    d.logT = ilog2ll(T);
     d.in_sn = in_sn, d.in_sc = in_sc, d.in_so = in_so;
     d.out_sk = out_sk, d.out_sc = out_sc, d.out_so = out_so;
     d.C = C;
-    d.tiles_per_o = (C + T - 1) / T;
-    d.ntiles = O * d.tiles_per_o;
     d.in_tfast = in_tfast ? 1 : 0;
     d.out_tfast = out_tfast ? 1 : 0;
     d.ptw = ptw ? 1 : 0;
     d.scale = 1.0f;
     p.async_ok = false;
-    p.smem = (size_t)(c.buf[0] + c.buf[1] + c.ptw) * sizeof(float2);
+    p.smem = uneven_tiles(d, c, O);
     p.grid = 0;  // launched through its phase's launch only
     return FB_FFT_OK;
 }
@@ -1610,6 +1617,9 @@ int recipe_create(BatchRecipe** out, int rank, const long long* dims, long long 
         j.dst = q.dst == kBufOut ? 1 : 2;
         j.last = q.last;
         j.smem = q.smem;
+        j.narrow = j.d;
+        j.narrow_smem = uneven_tiles(j.narrow, uneven_shape(q.d.L, q.d.C, q.io, kUnevenNarrowCap),
+                                     q.d.ntiles / q.d.tiles_per_o);
         r->jobs.push_back(j);
         r->phases = std::max(r->phases, q.group + 1);
         r->tiles += q.d.ntiles;

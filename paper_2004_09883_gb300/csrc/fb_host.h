@@ -34,6 +34,9 @@ struct BatchJob {
     int src, dst;     // 0 the request's input, 1 its output, 2 its scratch
     bool last;        // the job that finishes the transform (takes the 1/N scale)
     size_t smem;      // shared memory its tiles need (bytes)
+    // The same job in narrower tiles (same bits), for launches of few tiles
+    UnevenDesc narrow;
+    size_t narrow_smem;
 };
 // A four-step request whose strided tiles would move rows of fewer values than
 // kBatchRows (64 bytes; factors above 512 points) and which has at least

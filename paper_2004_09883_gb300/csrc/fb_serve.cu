@@ -164,6 +164,7 @@ struct Slot {
 struct fb_fft_server_s {
     uint32_t magic = kServerMagic;
     int device = 0;
+    int sms = 0;
     int max_plans = 1;
     std::chrono::steady_clock::time_point t0;
     cudaStream_t build = nullptr;  // plans are built here
@@ -374,6 +375,13 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
         for (int dir = 0; dir < 2; ++dir) {
             const bool fwd = dir == 0;
             Group g{fwd, nj, 0, nt, 0, 0};
+            // fewer tiles than SMs: narrower ones (kUnevenNarrowCap)
+            long long wide = 0;
+            for (const Req& r : sl.reqs)
+                if ((r.direction == FB_FFT_FORWARD) == fwd)
+                    for (const host::BatchJob& j : r.pe->recipe->jobs)
+                        if (j.phase == ph) wide += j.d.ntiles;
+            const bool narrow = wide < s->sms;
             for (size_t i = 0; i < sl.reqs.size(); ++i) {
                 const Req& r = sl.reqs[i];
                 if ((r.direction == FB_FFT_FORWARD) != fwd) continue;
@@ -389,7 +397,7 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
                 for (const host::BatchJob& j : r.pe->recipe->jobs) {
                     if (j.phase != ph) continue;
                     UnevenDesc& d = jobs[nj];
-                    d = j.d;
+                    d = narrow ? j.narrow : j.d;
                     d.in = j.src == 0 ? in : (j.src == 1 ? out : scratch);
                     d.out = j.dst == 1 ? out : scratch;
                     d.in_buf = 3;
@@ -397,8 +405,8 @@ int start_batch(fb_fft_server_s* s, Slot& sl)
                     d.err = sl.err_dev;
                     d.apply_scale = (j.last && scale) ? 1 : 0;
                     tiles[nt++] = (int)g.ntiles;
-                    g.ntiles += j.d.ntiles;
-                    g.smem = std::max(g.smem, j.smem);
+                    g.ntiles += d.ntiles;
+                    g.smem = std::max(g.smem, narrow ? j.narrow_smem : j.smem);
                     ++nj;
                     ++g.njobs;
                 }
@@ -589,6 +597,7 @@ int fb_fft_server_create(fb_fft_server_t* srv, int slots, long long hbm_cap_byte
     if (!s) return FB_FFT_ERR_ALLOC;
     s->t0 = std::chrono::steady_clock::now();
     cudaGetDevice(&s->device);
+    cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, s->device);
     s->max_plans = max_plans;
     s->slots.resize(slots);
     s->st.slots = slots;

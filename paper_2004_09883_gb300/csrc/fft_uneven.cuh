@@ -39,6 +39,12 @@ namespace fbfft {
 constexpr int kUnevenThreads = 256;
 constexpr int kUnevenCtas = 3;        // per SM: 72 registers, 70 KB of exchange buffers
 constexpr int kUnevenCap = 4096;      // values per tile
+// ... and of a server launch whose tiles would not even give every SM one: twice as
+// many SMs work then.  Lone requests, us on the device with tiles of 4096 / 2048 /
+// 1024 values: 512 x 512 22.3 / 18.7 / 18.5, 2^18 22.7 / 19.1 / 19.4, 256 x 256 19.0 /
+// 16.0 / 15.8, 16384 16.7 / 15.3 / 15.2; once there is a tile for every SM the wide ones
+// win (8 requests of 2^19: 69 against 80 us).
+constexpr int kUnevenNarrowCap = 2048;
 constexpr int kUnevenMaxLen = 2048;   // longest line of a job
 constexpr int kUnevenMaxRadix = 16;
 constexpr int kUnevenMaxLines = 128;  // contiguous lines per tile
@@ -610,17 +616,17 @@ inline const MrSchedule& uneven_schedule(int L, bool contiguous)
 }
 
 // Lines per tile of a job of L-point lines (C per outer index): as many as fit
-// 4096 values -- any number of contiguous lines (at most 128), a power of two
+// `cap` values -- any number of contiguous lines (at most 128), a power of two
 // where a side is strided (rows of T consecutive values: 16, or 32 for short
 // lines, whatever fits).
-inline int uneven_lines(long long L, long long C, int io)
+inline int uneven_lines(long long L, long long C, int io, int cap = kUnevenCap)
 {
     auto floor2 = [](long long x) {
         long long p = 1;
         while (p * 2 <= x) p *= 2;
         return p;
     };
-    long long T = std::max(1LL, kUnevenCap / L);
+    long long T = std::max(1LL, cap / L);
     if (io == 0)  // contiguous on both sides
         T = std::min<long long>(std::min<long long>(T, kUnevenMaxLines), C);
     else
@@ -630,7 +636,7 @@ inline int uneven_lines(long long L, long long C, int io)
 
 // Shape of such a job on the one-kernel batched-uneven engine: the
 // composite-radix schedule of radices up to 16, and uneven_lines per tile.
-inline MrConfig uneven_shape(long long L, long long C, int io)
+inline MrConfig uneven_shape(long long L, long long C, int io, int cap = kUnevenCap)
 {
     MrConfig c{};
     c.L = (int)L, c.io = io;
@@ -641,7 +647,7 @@ inline MrConfig uneven_shape(long long L, long long C, int io)
         c.ns[i] = ns;
         ns *= c.radix[i];
     }
-    c.T = uneven_lines(L, C, io);
+    c.T = uneven_lines(L, C, io, cap);
     return c;
 }
 

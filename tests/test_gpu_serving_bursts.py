@@ -57,3 +57,23 @@ def test_large_long_requests_run_their_plan(fb, n, batch):
     alone, _, one = burst(fb, n, batch, 1, INV)
     assert one == 2 and torch.equal(alone[0], ys[0])
     check(fb, ys[2], xs[2], n, batch, INV)
+
+
+@pytest.mark.parametrize("dims,counts", [((512, 512), (1, 2, 3)), ((1 << 18,), (1, 2, 3)), ((100, 100), (1, 16)),
+                                         ((16384,), (1, 37, 38)), ((64, 64, 64), (1, 2, 3)), ((45, 24, 50), (1, 7)),
+                                         ((2048,), (1, 64)), ((60,), (1, 64)), ((157464,), (1, 2, 4)),
+                                         ((3, 1000), (1, 20))])
+@pytest.mark.parametrize("direction", [FWD, INV])
+def test_narrow_and_wide_tiles_give_the_same_bits(fb, dims, counts, direction):
+    """Launches of fewer tiles than the GPU has SMs run in narrower tiles: the same
+    request alone, in bursts on both sides of that limit, and against the oracle."""
+    import torch
+    first = None
+    for count in counts:
+        ys, xs, _ = burst(fb, dims, 1, count, direction)
+        first = ys[0] if first is None else first
+        assert torch.equal(first, ys[0]), count
+        n = int(np.prod(dims))
+        ref = oracle.fft(xs[-1].cpu().numpy().astype(np.complex128), list(dims), direction, False, 8)
+        err = oracle.rel_l2(ys[-1].cpu().numpy().reshape(1, n), ref.reshape(1, n)).max()
+        assert err <= 2e-6 * np.log2(n), (dims, count, err)
