@@ -465,7 +465,7 @@ __device__ __forceinline__ void udeps_wait(const UnevenArgs& a, int dep, int nee
 template <bool FWD, bool INL, bool ONE>
 __device__ __forceinline__ void uneven_body(const UnevenArgs& a, const UnevenDesc* jobs, const int* tile_start)
 {
-    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    extern __shared__ __align__(128) unsigned char smem_dyn[];
     float2* buf = reinterpret_cast<float2*>(smem_dyn);
     __shared__ UnevenDesc sd[2];  // the descriptors of two tiles in turn
     __shared__ UTile s_tile[2];
