@@ -159,15 +159,17 @@ template <int R>
 struct UTwiddle {
     static constexpr int N = R <= 6 ? (R > 1 ? R - 1 : 1) : 1 + (R - 1) / 4;
     float2 w[N];
+    // the power of w that w[m] holds
+    __host__ __device__ static constexpr int power(int m) { return R <= 6 ? m + 1 : (m ? 4 * m : 1); }
     __device__ __forceinline__ void load(const float2* tw, int Ns)  // tw: the table at k
     {
         if constexpr (R > 1) {
 #pragma unroll
-            for (int m = 0; m < N; ++m) w[m] = __ldg(tw + (R <= 6 ? m : (m ? 4 * m - 1 : 0)) * Ns);
+            for (int m = 0; m < N; ++m) w[m] = __ldg(tw + (power(m) - 1) * Ns);
         }
     }
     template <bool FWD>
-    __device__ __forceinline__ void apply(float2* v) const
+    __host__ __device__ __forceinline__ void apply(float2* v) const
     {
         if constexpr (R <= 6) {
 #pragma unroll
