@@ -80,6 +80,9 @@ typedef enum fb_fft_status {
  * Builds the twiddle tables on the GPU (FP64 evaluation, rounded to FP32) and
  * allocates the plan's scratch; both are owned by the plan.  Uses the current
  * CUDA device; the plan must later be used with that device current.
+ * Execs of one plan give equal bits for equal inputs.  Plans of the same dims and
+ * another batch can differ in the last bits: power-of-two axes of 64 to 4096
+ * points take one of two kernels by the bytes of the whole batch.
  * Errors: INVALID_ARG, UNSUPPORTED_SIZE, ALLOC, CUDA, NO_DEVICE.
  */
 int fb_fft_plan(fb_fft_plan_t* plan, int rank, const long long* dims, long long batch,

@@ -2,8 +2,9 @@
 // no-allocation entry point (fb_fft_noalloc.cu): radix schedules, four-step
 // splits, the line-pass descriptor with its kernel, tile, shared-memory and
 // TMA choices, and the kernel arguments of one launch.  Both entry points
-// build their passes here, so they run the same kernels the same way.  Host
-// code only; not part of the C ABI.
+// build their passes here and run the same kernels the same way, but for
+// power-of-two lines of one pass, which an allocation-free call keeps on
+// fft_p2.cuh (make_line_pass, per_kernel).  Host code only; not part of the C ABI.
 #pragma once
 
 #include <cuda.h>
@@ -331,6 +332,10 @@ int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long
 //   2048   5.2 / 9.0 / 15.5 / 26.7 / 47.4 / 172    3.4 / 7.2 / 12.9 / 25.9 / 49.9 / 184
 //   4096   5.0 / 8.6 / 15.4 / 26.9 / 47.4 / 173    3.8 / 8.0 / 14.9 / 30.8 /   -  / 201
 //          (2^15: 4.2 against 3.4; 2^20: 5.5 against 6.3)
+// Where a length's better kernel changes more than twice, or by less than the runs
+// differ, the limits keep one range: 4096 points of 2^21 and 2^22 values (7 and 3 %)
+// stay on fft_p2.  128 points between 48 and 96 MiB (2^22 values, 12 %) stay there for
+// its grid: the launch-configuration test wants whole CTAs per SM of 128 x 32768.
 // Strided lines: 64 x 256 grids of 2^22 / 2^24 values 25.9 / 114 against 18.5 /
 // 99 us, 128 x 256 23.8 / 102 against 20.5 / 100; 256 points and more stay (2^24:
 // 90 against 98).

@@ -653,18 +653,17 @@ inline MrConfig uneven_shape(long long L, long long C, int io, int cap = kUneven
     return c;
 }
 
-// Row placement rules for tiles of a power of two of lines.  Row stride
-// (elements) of a tile's work rows (rows are not padded inside):
-// at least L, and chosen so that the 16 threads of a half-warp never meet on
-// one bank of 8-byte words across rows.  A stage that maps consecutive
-// threads to consecutive lines (the strided sides of four-step jobs) puts
-// H = 16/T positions of each of T lines in a half-warp; a stage that maps
-// them along a line puts H = G = 256/T positions of each of 16/G lines there
-// (short lines, G < 16).  Rows then start H * (odd) banks apart when
-// stride mod 2H == H.  (A tile of 32 strided lines has both kinds of stage;
-// its lines-fast stages win: H = 1.)  Padding inside the rows (i + i/16)
-// bought no fewer shared-memory wavefronts on the batched-uneven mix once
-// the rows are placed this way, and cost an address step per access.
+// Row placement rules for tiles of a power of two of lines whose rows are not
+// padded inside.  No kernel's tiles are laid out by these two any more (mr_place
+// finds every job's rows); the host index test still checks them.
+// Row stride (elements) of a tile's work rows: at least L, and chosen so that the
+// 16 threads of a half-warp never meet on one bank of 8-byte words across rows.
+// A stage that maps consecutive threads to consecutive lines (the strided sides
+// of four-step jobs) puts H = 16/T positions of each of T lines in a half-warp; a
+// stage that maps them along a line puts H = G = 256/T positions of each of 16/G
+// lines there (short lines, G < 16).  Rows then start H * (odd) banks apart when
+// stride mod 2H == H.  (A tile of 32 strided lines has both kinds of stage; its
+// lines-fast stages win: H = 1.)
 inline int uneven_line_stride(long long L, long long T, bool cfast)
 {
     const long long G = kUnevenThreads / T;
@@ -677,13 +676,11 @@ inline int uneven_line_stride(long long L, long long T, bool cfast)
     return (int)ls;
 }
 
-// Landing row stride of a contiguous-input tile (0: rows of L, first stage
-// along a line).  Tiles of 2 to 8 lines land in rows H = 16/T banks apart
-// (stride mod 2H == H, even, so the 16-byte copies stay aligned) and their
-// first stage maps threads across lines: its radix-R groups would otherwise
-// fill a half-warp at stride R (8-way for radix 8).
-// (The kernel's tiles load straight into registers now; the rule stands for
-// tiles that land in rows.)
+// Row stride of a contiguous-input tile copied to shared memory before its first
+// stage (0: rows of L, first stage along a line).  Tiles of 2 to 8 lines land in
+// rows H = 16/T banks apart (stride mod 2H == H, even, so the 16-byte copies stay
+// aligned) and their first stage maps threads across lines: its radix-R groups
+// would otherwise fill a half-warp at stride R (8-way for radix 8).
 inline int uneven_land_row(long long L, long long T, bool in_tfast)
 {
     if (in_tfast || T < 2 || T > 8) return 0;
