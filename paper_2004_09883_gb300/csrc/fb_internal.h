@@ -208,8 +208,9 @@ long long plane_smem_bytes(int lg1, int lg2, int threads);
 // Clusters of a cluster kernel that fit the GPU at once.
 cudaError_t line_cluster_occupancy(const LineKernel& k, size_t smem, int* clusters);
 LineKernel line_kernel_mixed(bool forward, int lg2);
-// Composite-radix pass (fft_mr.cuh) of L points, io = its IoMode.
-LineKernel line_kernel_mr(bool forward, int L, int io);
+// Composite-radix pass (fft_mr.cuh) of L points, io = its IoMode; fold: in tiles of
+// several outer indices (PassDesc::fold).
+LineKernel line_kernel_mr(bool forward, int L, int io, bool fold = false);
 // Raise a kernel's dynamic shared-memory limit to the device's opt-in maximum,
 // once per (kernel, device); split_regs > 0 also checks the kernel's register
 // count (see LineKernel::split_regs).

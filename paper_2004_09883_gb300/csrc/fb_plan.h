@@ -200,7 +200,7 @@ inline LineKernel pass_kernel(const PassPlan& q, bool fwd)
     }
     if (q.tc) return line_kernel_p2tc(q.threads, fwd, q.lg, q.io);
     if (q.kind == 3) return line_kernel_plane(fwd, q.lg1, q.lg, q.threads);
-    if (q.kind == 5) return line_kernel_mr(fwd, q.d.L, q.io);
+    if (q.kind == 5) return line_kernel_mr(fwd, q.d.L, q.io, q.d.fold != 0);
     if (q.kind == 2) return line_kernel_mixed(fwd, q.lg);
     if (q.kind == 1) return line_kernel_generic(fwd);
     return line_kernel_p2(q.threads, fwd, q.lg, q.io);

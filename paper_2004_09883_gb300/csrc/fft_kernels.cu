@@ -53,17 +53,19 @@ FB_MR_DECL(nn)
 FB_MR_DECL(cc)
 FB_MR_DECL(nc)
 FB_MR_DECL(ccp)
+FB_MR_DECL(fold)
 #undef FB_MR_DECL
-LineKernel line_kernel_mr(bool forward, int L, int io)
+LineKernel line_kernel_mr(bool forward, int L, int io, bool fold)
 {
     using Table = LineKernel (*)(int);
 #define FB_MR_TABLES(IO) \
     {line_kernel_mr_fwd_##IO##_a, line_kernel_mr_fwd_##IO##_b, line_kernel_mr_inv_##IO##_a, line_kernel_mr_inv_##IO##_b}
-    static const Table tables[4][4] = {FB_MR_TABLES(nn), FB_MR_TABLES(cc), FB_MR_TABLES(nc), FB_MR_TABLES(ccp)};
+    static const Table tables[5][4] = {FB_MR_TABLES(nn), FB_MR_TABLES(cc), FB_MR_TABLES(nc), FB_MR_TABLES(ccp),
+                                       FB_MR_TABLES(fold)};
 #undef FB_MR_TABLES
     LineKernel k{nullptr, 0, false, 0, 0};
-    if (io < 0 || io > 3) return k;
-    for (int half = 0; half < 2 && !k.fn; ++half) k = tables[io][(forward ? 0 : 2) + half](L);
+    if (io < 0 || io > 3 || (fold && io != kIoCC)) return k;
+    for (int half = 0; half < 2 && !k.fn; ++half) k = tables[fold ? 4 : io][(forward ? 0 : 2) + half](L);
     return k;
 }
 

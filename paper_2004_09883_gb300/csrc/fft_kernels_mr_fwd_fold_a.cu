@@ -1,0 +1,20 @@
+// fft_kernels_mr_fwd_fold_a.cu -- composite-radix line passes, forward:
+// strided lines in tiles of several outer indices.
+#include "fft_p2.cuh"
+#include "fft_mr.cuh"
+#include "mr_lengths.h"
+
+namespace fbfft {
+
+LineKernel line_kernel_mr_fwd_fold_a(int L)
+{
+    switch (L) {
+#define FB_MR_CASE(N) \
+    case N: return mr_fold_entry<true, N>();
+        FB_MR_LENGTHS_A(FB_MR_CASE)
+        FB_MR_POW2_CC(FB_MR_CASE)
+    default: return LineKernel{nullptr, 0, false, 0, 0};
+    }
+}
+
+}  // namespace fbfft

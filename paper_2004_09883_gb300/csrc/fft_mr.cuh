@@ -188,11 +188,18 @@ __device__ __forceinline__ float2 mr_ptw(const PassDesc& d, unsigned m)
     return cmul(__ldg(d.ptw_hi + (m >> d.ptw_log)), __ldg(d.ptw_lo + (m & ((1u << d.ptw_log) - 1))));
 }
 
+// How a tile's strided sides move: by its threads, by TMA, or by its threads with
+// the lines of several outer indices in the tile (PassDesc::fold).  The last is a
+// kernel of its own: as a run-time case of the first the line's address cost the
+// short strided lines 5 to 19 % (216 points 22.0 -> 26.1 us at 2^23 values).
+enum MrMode { kMrPlain = 0, kMrCopied = 1, kMrFold = 2 };
+
 // Where line t of a strided tile starts relative to its first line (so: values
 // between outer indices).
+template <int MODE>
 __device__ __forceinline__ long long mr_line(const PassDesc& d, int t, long long so)
 {
-    if (d.fold == 0) return t;
+    if constexpr (MODE != kMrFold) return t;
     const int o = (int)((unsigned)t * d.fold_mag >> 16);
     return o * so + (t - o * d.fold);
 }
@@ -204,13 +211,14 @@ struct Mr {
     static_assert(c.n >= 2, "no schedule");
 };
 
-// Stage S of the tile whose first line starts at gin / gout.  COPIED: the strided
+// Stage S of the tile whose first line starts at gin / gout.  kMrCopied: the strided
 // sides of the tile are in buf0 (dense, [position][line]), moved by TMA.
-template <bool FWD, int L, int IO, bool COPIED, int S>
+template <bool FWD, int L, int IO, int MODE, int S>
 __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, float2* gout, float2* buf0,
                                          float2* buf1, float2* ptw, int Tv, int c0, unsigned long long pol)
 {
     constexpr MrConfig C = Mr<L, IO>::c;
+    constexpr bool COPIED = MODE == kMrCopied;
     constexpr bool first = S == 0, last = S == C.n - 1;
     constexpr bool IN_T = Mr<L, IO>::IN_T, OUT_T = Mr<L, IO>::OUT_T, tfast = first ? IN_T : OUT_T;
     constexpr int R = C.radix[S], LR = L / R, Ns = C.ns[S], TH = C.threads;
@@ -255,7 +263,7 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
 #pragma unroll
                 for (int r = 0; r < R; ++r) v[u][r] = p[r * LR * C.T];
             } else if constexpr (first) {
-                const float2* p = IN_T ? gin + (long long)j[u] * d.in_sn + (IO == 1 ? mr_line(d, t[u], d.in_so) : t[u])
+                const float2* p = IN_T ? gin + (long long)j[u] * d.in_sn + mr_line<MODE>(d, t[u], d.in_so)
                                        : gin + t[u] * L + j[u];
                 long long step = IN_T ? LR * d.in_sn : LR;
                 if constexpr (IO == 2) {
@@ -291,7 +299,7 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
                 for (int r = 0; r < R; ++r) p[r * Ns] = v[u][r];
             } else {
                 // Ns = L / R: the outputs of butterfly j are j + r Ns
-                float2* p = OUT_T ? gout + (long long)j[u] * d.out_sk + (IO == 1 ? mr_line(d, t[u], d.out_so) : t[u])
+                float2* p = OUT_T ? gout + (long long)j[u] * d.out_sk + mr_line<MODE>(d, t[u], d.out_so)
                                   : gout + t[u] * L + j[u];
                 const long long step = OUT_T ? Ns * d.out_sk : Ns;
                 if constexpr (IO == 3) {
@@ -333,19 +341,19 @@ __device__ __forceinline__ void mr_stage(const PassDesc& d, const float2* gin, f
     }
 }
 
-template <bool FWD, int L, int IO, bool COPIED>
+template <bool FWD, int L, int IO, int MODE>
 __device__ __forceinline__ void mr_tile(const PassDesc& d, const float2* gin, float2* gout, float2* buf0,
                                         float2* buf1, float2* ptw, int Tv, int c0, unsigned long long pin,
                                         unsigned long long pout)
 {
     constexpr int n = Mr<L, IO>::c.n;
-    mr_stage<FWD, L, IO, COPIED, 0>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pin);
-    mr_stage<FWD, L, IO, COPIED, 1>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
-    if constexpr (n > 2) mr_stage<FWD, L, IO, COPIED, 2>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
-    if constexpr (n > 3) mr_stage<FWD, L, IO, COPIED, 3>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
+    mr_stage<FWD, L, IO, MODE, 0>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pin);
+    mr_stage<FWD, L, IO, MODE, 1>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
+    if constexpr (n > 2) mr_stage<FWD, L, IO, MODE, 2>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
+    if constexpr (n > 3) mr_stage<FWD, L, IO, MODE, 3>(d, gin, gout, buf0, buf1, ptw, Tv, c0, pout);
 }
 
-template <bool FWD, int L, int IO>
+template <bool FWD, int L, int IO, bool FOLD = false>
 __global__ void __maxnreg__((Mr<L, IO>::c.regs)) k_fft_mr(const __grid_constant__ LineArgs a)
 {
     extern __shared__ __align__(128) unsigned char mr_smem_dyn[];
@@ -358,7 +366,7 @@ __global__ void __maxnreg__((Mr<L, IO>::c.regs)) k_fft_mr(const __grid_constant_
     float2* buf0 = reinterpret_cast<float2*>(mr_smem + 128);
     float2* buf1 = buf0 + C.buf[0];
     float2* ptw = buf1 + C.buf[1];
-    const bool copied = C.in_place && d.async_io != 0;
+    const bool copied = !FOLD && C.in_place && d.async_io != 0;
     if constexpr (IN_T) {
         if (copied) {
             if (threadIdx.x == 0) {
@@ -406,10 +414,11 @@ __global__ void __maxnreg__((Mr<L, IO>::c.regs)) k_fft_mr(const __grid_constant_
                 phase ^= 1u;
             }
         }
-        if (C.in_place && copied)
-            mr_tile<FWD, L, IO, C.in_place>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pin, pout);
+        if (!FOLD && C.in_place && copied)
+            mr_tile<FWD, L, IO, !FOLD && C.in_place ? kMrCopied : kMrPlain>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0,
+                                                                             pin, pout);
         else
-            mr_tile<FWD, L, IO, false>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pin, pout);
+            mr_tile<FWD, L, IO, FOLD ? kMrFold : kMrPlain>(d, gin, gout, buf0, buf1, ptw, Tv, (int)c0, pin, pout);
         if constexpr (OUT_T) {
             if (copied) {
                 fence_proxy_async();  // the tile -> visible to the copy engine
@@ -432,13 +441,23 @@ __global__ void __maxnreg__((Mr<L, IO>::c.regs)) k_fft_mr(const __grid_constant_
     }
 }
 
-template <bool FWD, int L, int IO>
+template <bool FWD, int L, int IO, bool FOLD = false>
 LineKernel mr_entry()
 {
-    LineKernel k = make_entry<Mr<L, IO>::c.threads>(k_fft_mr<FWD, L, IO>, FWD, L, IO);
+    LineKernel k = make_entry<Mr<L, IO>::c.threads>(k_fft_mr<FWD, L, IO, FOLD>, FWD, L, IO);
     k.kind = 5;
     k.mr = &Mr<L, IO>::c;
     return k;
+}
+// Strided lines in tiles of several outer indices: lengths whose tiles hold two
+// outer indices of two lines and more.
+template <bool FWD, int L>
+LineKernel mr_fold_entry()
+{
+    if constexpr (Mr<L, 1>::c.T >= 4)
+        return mr_entry<FWD, L, 1, true>();
+    else
+        return LineKernel{nullptr, 0, false, 0, 0};
 }
 
 #endif  // __CUDACC__
