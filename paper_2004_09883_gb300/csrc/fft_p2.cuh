@@ -134,6 +134,8 @@ struct P2 {
     static constexpr bool IN_T = io_in_strided(IO);
     static constexpr bool OUT_T = io_out_strided(IO);
     static constexpr bool PTW = IO == kIoCCP;
+    // Tensor-core stages: twiddles read ahead of their barrier (p2_tc_twiddles)
+    static constexpr bool TW_AHEAD = PTW || (IO == kIoNC && LG >= 11);
     static constexpr int T = p2_tile_lines(THREADS, LG, IO);
     static constexpr int LOGT = ilog2(T);
     static constexpr int G = THREADS / T;
@@ -397,7 +399,8 @@ __device__ __forceinline__ void p2_stage_tc(const PassDesc& d, float2* land, flo
     const int k = j & (NS - 1);
     if constexpr (NS > 1) {
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = twmul<FWD>(v[r], twr[r - 1]);
+        for (int r = 1; r < R; ++r)
+            v[r] = twmul<FWD>(v[r], C::TW_AHEAD ? twr[r - 1] : __ldg(d.tw + d.twoff[S] + k + (r - 1) * NS));
     }
     const unsigned abase = smem_u32(work);
     int e;
@@ -452,13 +455,18 @@ __device__ __forceinline__ void p2_stage_tc(const PassDesc& d, float2* land, flo
 }
 
 // The twiddles of tensor-core stage S (global memory, L1-cached: a CTA's tables
-// do not fit beside two CTAs' tiles), read ahead of the barrier before it.
+// do not fit beside two CTAs' tiles), read ahead of the barrier before it where the
+// stage waits longest for its tile: four-step columns (2^20 x 32 with the factor
+// table 287 us, without either 308) and rows of 2048 points (2^22 x 2 107 -> 98 us;
+// shorter rows lose 2 to 3 %, 2^20 x 32 282 -> 288).  Elsewhere the 30 registers cost
+// more than the wait: contiguous lines 3 to 8 % (4096 x 16384 279 -> 301 us, 512 x
+// 131072 233 -> 251), strided lines 2 to 5 % (4096 x 4096 393 -> 409).
 template <int THREADS, int LG, int IO, int S>
 __device__ __forceinline__ void p2_tc_twiddles(const PassDesc& d, float2 (&twr)[15])
 {
-    if constexpr (S < pow2_nst(LG)) {
+    using C = P2<THREADS, LG, IO>;
+    if constexpr (C::TW_AHEAD && S < pow2_nst(LG)) {
         if constexpr (pow2_radix(LG, S) == 16 && pow2_ns(LG, S) > 1) {
-            using C = P2<THREADS, LG, IO>;
             constexpr bool tfast = S == C::NST - 1 && C::OUT_T;
             constexpr int NS = pow2_ns(LG, S);
             const int j = tfast ? (int)(threadIdx.x >> C::LOGT) : (int)(threadIdx.x & (C::G - 1));
