@@ -770,6 +770,30 @@ long long fourstep_blocks(long long N1, long long N2)
     return (N2 / r->radix[0]) % a->T == 0 ? a->T : 0;
 }
 
+// MiB a pass reads and writes.
+long long pass_mib(const PassPlan& q)
+{
+    return (long long)q.d.L * q.d.C * (q.d.ntiles / std::max(1LL, q.d.tiles_per_o)) * 16 >> 20;
+}
+
+// Which passes start while the one before them drains (programmatic dependent
+// launch): all but those whose data exceed kMixedOverlapMib where one of the two is
+// a composite-radix pass (a CTA per tile, thousands of them) and the other is not
+// (persistent CTAs with most of an SM's shared memory): waiting CTAs of the one keep
+// the other from its SMs.  us per exec with and without the overlap: 4096 x 128 x 32
+// (256 MiB) 149 / 119, 256 x 1000 x 131 (512 MiB) 200 / 191, 512 x 360 x 91 (256 MiB) 115 /
+// 103, 64 x 256 x 256 x 4 (256 MiB) 148 / 133.  At 64 to 160 MiB it is the other way
+// round as often as not (1000 x 256 x 39, 158 MiB: 64 / 68; 256 x 240 x 165, 158 MiB: 60 / 54),
+// below that the overlap always gains (256 x 256 x 32, 32 MiB: 13 / 16.5).
+constexpr long long kMixedOverlapMib = 192;
+void overlap_passes(std::vector<PassPlan>& passes)
+{
+    for (size_t i = 0; i < passes.size(); ++i) {
+        const PassPlan& before = passes[i ? i - 1 : passes.size() - 1];  // (the last one: the exec before)
+        passes[i].overlap = (passes[i].kind == 5) == (before.kind == 5) || pass_mib(passes[i]) <= kMixedOverlapMib;
+    }
+}
+
 // Host part of planning: the pass list and the twiddle jobs (no device work).
 int schedule_plan(fb_fft_plan_s* p, TwiddleBuilder& twb)
 {
@@ -913,6 +937,7 @@ int build_plan(fb_fft_plan_s* p)
     FB_CK(cudaMemsetAsync(p->err, 0, 16 * sizeof(int), p->stream));
     int sms = 0;
     FB_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
+    if (!p->many) overlap_passes(p->passes);
     for (PassPlan& q : p->passes) {
         int occ = 0;
         const LineKernel k = pass_kernel(q, true);
@@ -1106,7 +1131,7 @@ int launch_pass(fb_fft_plan_s* p, const PassPlan& q, const float2* in, float2* o
         cudaEventRecord(e0, stream);
     }
     const LineKernel k = pass_kernel(q, fwd);
-    const cudaError_t le = line_launch(k, args, q.grid, smem, stream);
+    const cudaError_t le = line_launch(k, args, q.grid, smem, stream, q.overlap);
     if (le != cudaSuccess) {
         char nm[64];
         line_kernel_name(k, nm, sizeof(nm));

@@ -216,7 +216,9 @@ LineKernel line_kernel_mr(bool forward, int L, int io, bool fold = false);
 // count (see LineKernel::split_regs).
 cudaError_t kernel_smem_optin(const void* fn, int split_regs);
 // Launch / occupancy / name of a table entry (shared-memory opt-in handled inside).
-cudaError_t line_launch(const LineKernel& k, const LineArgs& a, long long grid, size_t smem, cudaStream_t stream);
+// overlap: the launch may start while the kernel before it on the stream drains.
+cudaError_t line_launch(const LineKernel& k, const LineArgs& a, long long grid, size_t smem, cudaStream_t stream,
+                        bool overlap = true);
 cudaError_t line_occupancy(const LineKernel& k, size_t smem, int* blocks_per_sm);
 void line_kernel_name(const LineKernel& k, char* buf, size_t n);
 

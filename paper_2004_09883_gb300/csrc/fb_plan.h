@@ -65,6 +65,7 @@ struct PassPlan {
     int lg1 = 0;
     long long grid;
     size_t smem;
+    bool overlap = true;  // the launch may start while the pass before it drains (overlap_passes)
     bool async_ok;  // tiles can move by TMA (given 16-byte aligned buffer bases)
     int src, dst;
     long long src_off, dst_off;  // element offsets into the source / destination buffer

@@ -131,7 +131,8 @@ bool pdl_enabled()
 cudaError_t ensure_smem_attr(const LineKernel& k) { return kernel_smem_optin((const void*)k.fn, k.split_regs); }
 }  // namespace
 
-cudaError_t line_launch(const LineKernel& k, const LineArgs& a, long long grid, size_t smem, cudaStream_t stream)
+cudaError_t line_launch(const LineKernel& k, const LineArgs& a, long long grid, size_t smem, cudaStream_t stream,
+                        bool overlap)
 {
     if (grid <= 0) return cudaSuccess;
     cudaError_t e = ensure_smem_attr(k);
@@ -147,7 +148,7 @@ cudaError_t line_launch(const LineKernel& k, const LineArgs& a, long long grid, 
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = overlap && pdl_enabled() ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (k.cluster > 1) {  // the grid is a whole number of clusters (the planner sizes it so)
