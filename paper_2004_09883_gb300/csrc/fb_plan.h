@@ -338,12 +338,14 @@ int make_mr_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long long
 // stay on fft_p2.  128 points between 48 and 96 MiB (2^22 values, 12 %) stay there for
 // its grid: the launch-configuration test wants whole CTAs per SM of 128 x 32768.
 // Strided lines: 64 x 256 grids of 2^22 / 2^24 values 25.9 / 114 against 18.5 /
-// 99 us, 128 x 256 23.8 / 102 against 20.5 / 100; 256 points and more stay (2^24:
-// 90 against 98).
-inline bool pow2_on_mr(long long L, long long elems, int io)
+// 84 us, 128 x 256 23.8 against 18.5; above 192 MiB the 128-point pass loses 4 to 15 %
+// (128 x 512, 2^24 values: 47 against 51 us a pass, 94 / 98 the grid), but not behind
+// the short lines of a small trailing extent (128 x 32: 127 / 105 the grid); 256 points
+// and more stay (2^24: 90 against 98).  C: lines per outer index.
+inline bool pow2_on_mr(long long L, long long elems, int io, long long C)
 {
     const long long mib = 16 * elems >> 20;  // read and written
-    if (io == kIoCC) return L == 64 || L == 128;
+    if (io == kIoCC) return L == 64 || (L == 128 && (mib <= 192 || C < 64));
     if (io != kIoNN) return false;
     switch (L) {
     case 64: return mib <= 96 || mib > 192;
@@ -378,7 +380,7 @@ int make_line_pass(PassPlan& p, Twiddles& twb, long long L, long long O, long lo
     // 144 x 4 volume forward and back)
     const int io = ptw ? kIoCCP : (in_tfast ? kIoCC : (out_tfast ? kIoNC : kIoNN));
     const bool tc_pass = tc && pow2_len && line_kernel_p2tc(256, true, ilog2ll(L), io).fn != nullptr;
-    const bool on_mr = !pow2_len || (!tc_pass && pow2_on_mr(L, route_elems > 0 ? route_elems : O * C * L, io));
+    const bool on_mr = !pow2_len || (!tc_pass && pow2_on_mr(L, route_elems > 0 ? route_elems : O * C * L, io, C));
     if (on_mr && !per_kernel)
         return make_mr_pass(p, twb, L, O, C, in_sn, in_sc, in_so, out_sk, out_sc, out_so, in_tfast, out_tfast, ptw);
     p = PassPlan{};  // zero descriptor, default member values (no offset tables)

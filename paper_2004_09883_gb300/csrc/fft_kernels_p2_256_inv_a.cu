@@ -1,5 +1,5 @@
 // fft_kernels_p2_256_inv_a.cu -- 256-thread power-of-two line passes, inverse (exponent sign +1),
-// layouts: kIoNN kIoCC (strided lines of 64 and 128 points run on fft_mr.cuh).
+// layouts: kIoNN kIoCC (strided lines of 64 points run on fft_mr.cuh).
 #include "fft_p2.cuh"
 
 namespace fbfft {
@@ -19,6 +19,7 @@ LineKernel line_kernel_p2_256_inv_a(int lg, int io)
     case 5 * 4 + kIoCC: return p2_entry<256, false, 5, kIoCC>();
     case 6 * 4 + kIoNN: return p2_entry<256, false, 6, kIoNN>();
     case 7 * 4 + kIoNN: return p2_entry<256, false, 7, kIoNN>();
+    case 7 * 4 + kIoCC: return p2_entry<256, false, 7, kIoCC>();
     case 8 * 4 + kIoNN: return p2_entry<256, false, 8, kIoNN>();
     case 8 * 4 + kIoCC: return p2_entry<256, false, 8, kIoCC>();
     case 9 * 4 + kIoNN: return p2_entry<256, false, 9, kIoNN>();
