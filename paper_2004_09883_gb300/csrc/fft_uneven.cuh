@@ -17,11 +17,12 @@
 // one or two shared-memory buffers, stores straight back.  A control warp beside
 // the eight compute warps walks the job table one tile ahead.
 //
-// What bounds it: latency (issue slots 36 % busy, long scoreboard and barrier
-// stalls; 72 registers leave three CTAs per SM).  On 4096 lengths in [64, 65536]
-// the large radices halved the instructions (417 -> 206 M warp instructions, 180
-// -> 89 per value and pass) and took 565 -> 530 us; with the table walk, claims and
-// counter traffic moved to the control warp 418 us.  256 waiting requests of a
+// What bounds it: latency (issue slots 36 % busy; per issue 5.8 warps wait for
+// global loads, 4.0 at barriers; 72 registers leave three CTAs per SM).  On 4096
+// lengths in [64, 65536] the large radices and the control warp more than halved the
+// instructions (417 -> 188 M warp instructions, 166 -> 75 thread instructions per
+// value and pass): the radices took 565 -> 530 us, the table walk, claims and
+// counter traffic on the control warp 530 -> 418 us.  256 waiting requests of a
 // server, 2190 -> 1650 us: there the strided tiles of 1000- to 2048-point lines
 // (rows of 2 to 4 values) take most of the time.  Measured without gain: 128
 // compute threads and 2048 values per tile (420 us; the server's long lines then
