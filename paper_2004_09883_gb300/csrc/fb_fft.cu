@@ -779,8 +779,9 @@ long long pass_mib(const PassPlan& q)
 // Which passes start while the one before them drains (programmatic dependent
 // launch): all but those whose data exceed kMixedOverlapMib where one of the two is
 // a composite-radix pass (a CTA per tile, thousands of them) and the other is not
-// (persistent CTAs with most of an SM's shared memory): waiting CTAs of the one keep
-// the other from its SMs.  us per exec with and without the overlap: 4096 x 128 x 32
+// (persistent CTAs with most of an SM's shared memory).  There the early starts cost
+// more than they hide, presumably because CTAs that wait keep the other kernel's off
+// their SMs.  us per exec with and without the overlap: 4096 x 128 x 32
 // (256 MiB) 149 / 119, 256 x 1000 x 131 (512 MiB) 200 / 191, 512 x 360 x 91 (256 MiB) 115 /
 // 103, 64 x 256 x 256 x 4 (256 MiB) 148 / 133.  At 64 to 160 MiB it is the other way
 // round as often as not (1000 x 256 x 39, 158 MiB: 64 / 68; 256 x 240 x 165, 158 MiB: 60 / 54),
